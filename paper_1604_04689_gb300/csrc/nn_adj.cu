@@ -8,11 +8,19 @@
 // conforming mesh this is the dual graph; a hex face split into two tet
 // triangles borders both tets.
 //
-// One thread per element merges the (sorted) element rows of its distinct
-// nodes, which yields every element sharing a node with it once, in
-// ascending order, with the number of shared nodes; the face tests run only
-// where that number allows a shared face.  Three kernels: count, exclusive
-// scan (decoupled lookback over tiles of elements), and write.
+// A mesh of one type is matched node by node (k_adj_match): the elements
+// around a node are held by the lanes of a group, and a lane compares the
+// faces of its element that contain the node with every other element there.
+// Each face is settled once, at its smallest node, and what lies across it
+// goes into one slot per element and face; the rows are the sorted slots.
+// Elements for which one slot per face is not enough (several elements across
+// a face, a face that lies in an element without being one of its faces,
+// repeated nodes, a node with very many elements) are flagged.  A flagged
+// element, and every element of a mixed mesh, merges the (sorted) element
+// rows of its distinct nodes, which yields every element sharing a node with
+// it once, in ascending order, with the number of shared nodes; the face
+// tests run only where that number allows a shared face.  Then count,
+// exclusive scan (decoupled lookback over tiles of elements), and write.
 #include "nn_device.cuh"
 
 namespace nn {
@@ -123,11 +131,292 @@ __device__ __forceinline__ void for_each_neighbour(const AdjParams& p, int64_t e
     }
 }
 
+// ------------------------------------------------- matching node by node
+// What bounds the merge above is divergence: measured on a 61^3 Kuhn grid, 5
+// of 32 lanes were active on average, and every element's node rows were
+// walked twice.  Matching per node gathers each element's nodes once per node
+// (n_conn gathers in all) and has no data-dependent branch but the rare match.
+// Whole call, GB300: 101^3 Kuhn grid 26.7 -> 1.7 ms, 161^3 111 -> 6.9 ms,
+// 129^3 hex grid 3.0 -> 0.94 ms, 2048^2 triangle grid 7.3 -> 1.4 ms.  The
+// groups have 8 lanes where a node has 4 to 8 elements, a warp for tets (24).
+constexpr int ADJ_LONG = 64;  // longest node row matched here; elements around a longer one are flagged
+
+template <int TYPE>
+struct AdjShape;
+// Q: the element's nodes other than the centre; F: its faces at the centre;
+// NF: its faces (slots); G: lanes of a group, at least the ordinary number of
+// elements around a node (a longer row takes several rounds).
+template <>
+struct AdjShape<NN_TRI> {
+    static constexpr int Q = 2, F = 2, NF = 3, G = 8;
+};
+template <>
+struct AdjShape<NN_QUAD> {
+    static constexpr int Q = 3, F = 2, NF = 4, G = 8;
+};
+template <>
+struct AdjShape<NN_TET> {
+    static constexpr int Q = 3, F = 3, NF = 4, G = 32;
+};
+template <>
+struct AdjShape<NN_HEX> {
+    static constexpr int Q = 7, F = 3, NF = 6, G = 8;
+};
+
+__device__ __forceinline__ void cond_swap(bool c, int32_t& a, int32_t& b) {
+    const int32_t x = c ? b : a, y = c ? a : b;
+    a = x;
+    b = y;
+}
+
+// Element e seen from its node v: the other nodes in a frame with v at the
+// origin, and the slot of each face at v.
+template <int TYPE>
+struct AdjFrame {
+    using S = AdjShape<TYPE>;
+    int32_t q[S::Q];
+    int local;  // v's place in the element (hex: in binary corner order)
+
+    // 0: not usable (invalid element, or v is none of its nodes), 1: fine, 2: a node repeats
+    __device__ __forceinline__ int load(const AdjParams& p, int64_t e, int32_t v) {
+        constexpr int NPE = S::Q + 1;
+        int32_t nd[NPE];
+        if (e < 0 || e >= p.n_elems) return 0;
+        if constexpr (TYPE == NN_TRI) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) nd[i] = __ldg(p.conn + 3 * e + i);
+        } else {
+            const int4 a = __ldg(reinterpret_cast<const int4*>(p.conn) + (NPE / 4) * e);
+            nd[0] = a.x; nd[1] = a.y; nd[2] = a.z; nd[3] = a.w;
+            if constexpr (NPE == 8) {
+                const int4 b = __ldg(reinterpret_cast<const int4*>(p.conn) + 2 * e + 1);
+                nd[4] = b.x; nd[5] = b.y; nd[6] = b.z; nd[7] = b.w;
+            }
+        }
+        bool in = true, rep = false;
+        local = -1;
+#pragma unroll
+        for (int i = 0; i < NPE; ++i) {
+            in = in && (uint32_t)nd[i] < (uint64_t)p.n_nodes;
+            if (nd[i] == v) local = i;
+#pragma unroll
+            for (int j = 0; j < i; ++j) rep = rep || nd[i] == nd[j];
+        }
+        if (!in || local < 0) return 0;
+        if constexpr (TYPE == NN_TRI) {
+            q[0] = local == 0 ? nd[1] : (local == 1 ? nd[2] : nd[0]);
+            q[1] = local == 0 ? nd[2] : (local == 1 ? nd[0] : nd[1]);
+        } else if constexpr (TYPE == NN_QUAD) {
+            // turned until v comes first
+            if (local & 1) {
+                const int32_t t = nd[0];
+                nd[0] = nd[1]; nd[1] = nd[2]; nd[2] = nd[3]; nd[3] = t;
+            }
+            cond_swap(local & 2, nd[0], nd[2]);
+            cond_swap(local & 2, nd[1], nd[3]);
+            q[0] = nd[1]; q[1] = nd[2]; q[2] = nd[3];
+        } else if constexpr (TYPE == NN_TET) {
+            q[0] = local == 0 ? nd[1] : nd[0];
+            q[1] = local <= 1 ? nd[2] : nd[1];
+            q[2] = local <= 2 ? nd[3] : nd[2];
+        } else {
+            // binary corner order (VTK order with 2, 3 and 6, 7 swapped), then
+            // reflected along each axis on which v lies at the far side
+            cond_swap(true, nd[2], nd[3]);
+            cond_swap(true, nd[6], nd[7]);
+            if ((local & 3) >= 2) local ^= 1;
+#pragma unroll
+            for (int a = 1; a < 8; a <<= 1)
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (!(i & a)) cond_swap(local & a, nd[i], nd[i | a]);
+#pragma unroll
+            for (int i = 1; i < 8; ++i) q[i - 1] = nd[i];
+        }
+        return rep ? 2 : 1;
+    }
+    // whether every other node of face f at v is above v (v is the face's smallest node)
+    __device__ __forceinline__ bool smallest(int f, int32_t v) const {
+        if constexpr (TYPE == NN_TRI) return q[f] > v;
+        else if constexpr (TYPE == NN_QUAD) return q[2 * f] > v;
+        else if constexpr (TYPE == NN_TET) return q[f == 0 ? 1 : 0] > v && q[f == 2 ? 1 : 2] > v;
+        else return f == 0 ? (q[0] > v && q[1] > v && q[2] > v)
+                           : (f == 1 ? (q[0] > v && q[3] > v && q[4] > v) : (q[1] > v && q[3] > v && q[5] > v));
+    }
+    // slot of face f at v, unique over the element's faces
+    __device__ __forceinline__ int slot(int f) const {
+        if constexpr (TYPE == NN_TRI) return f == 0 ? local : (local == 0 ? 2 : local - 1);
+        else if constexpr (TYPE == NN_QUAD) return f == 0 ? local : (local + 3) & 3;
+        else if constexpr (TYPE == NN_TET) return f + (f >= local ? 1 : 0);  // the node left out
+        else return f == 0 ? 4 + ((local >> 2) & 1) : (f == 1 ? 2 + ((local >> 1) & 1) : (local & 1));
+    }
+    // faces at v (bit f) whose nodes all lie in the element with frame y (also seen from v)
+    __device__ __forceinline__ uint32_t inside(const int32_t* y) const {
+        bool in[S::Q];
+#pragma unroll
+        for (int k = 0; k < S::Q; ++k) {
+            in[k] = false;
+            if ((TYPE == NN_QUAD && k == 1) || (TYPE == NN_HEX && k == 6)) continue;  // on no face at v
+#pragma unroll
+            for (int i = 0; i < S::Q; ++i) in[k] = in[k] || q[k] == y[i];
+        }
+        if constexpr (TYPE == NN_TRI) return (in[0] ? 1u : 0u) | (in[1] ? 2u : 0u);
+        else if constexpr (TYPE == NN_QUAD) return (in[0] ? 1u : 0u) | (in[2] ? 2u : 0u);
+        else if constexpr (TYPE == NN_TET)
+            return (in[1] && in[2] ? 1u : 0u) | (in[0] && in[2] ? 2u : 0u) | (in[0] && in[1] ? 4u : 0u);
+        else
+            return (in[0] && in[1] && in[2] ? 1u : 0u) | (in[0] && in[3] && in[4] ? 2u : 0u) |
+                   (in[1] && in[3] && in[5] ? 4u : 0u);
+    }
+    // whether face f at v is, as far as a look at the frames shows, a face of
+    // y too (simplices: always; a false "no" only costs the slow path)
+    __device__ __forceinline__ bool also_face_of(int f, const int32_t* y) const {
+        if constexpr (TYPE == NN_QUAD) {
+            return q[2 * f] == y[0] || q[2 * f] == y[2];
+        } else if constexpr (TYPE == NN_HEX) {
+            const int32_t a = f == 2 ? q[1] : q[0], b = f == 0 ? q[1] : q[3], d = f == 0 ? q[2] : (f == 1 ? q[4] : q[5]);
+            auto is = [&](int32_t ya, int32_t yb, int32_t yd) {
+                return d == yd && ((a == ya && b == yb) || (a == yb && b == ya));
+            };
+            return is(y[0], y[1], y[2]) || is(y[0], y[3], y[4]) || is(y[1], y[3], y[5]);
+        } else {
+            return true;
+        }
+    }
+};
+
+// One node per group of G lanes, one element of its row per lane (rows of
+// more than G elements: several rounds, the others read from memory).
+template <int TYPE>
+__global__ void __launch_bounds__(ADJ_THREADS) k_adj_match(AdjParams p) {
+    using S = AdjShape<TYPE>;
+    constexpr int G = S::G, PER = 32 / G;
+    const int lane = threadIdx.x & 31, gl = lane & (G - 1);
+    const int64_t warp = ((int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x) >> 5;
+    const int64_t step = ((int64_t)gridDim.x * ADJ_THREADS >> 5) * PER;
+    // one lane's findings: the element across each face at v, and how many there are
+    struct Found {
+        int32_t y[S::F];
+        int n[S::F];
+    };
+    auto compare = [&](const AdjFrame<TYPE>& x, int32_t v, int32_t ey, const int32_t* y, Found& r) {
+        const uint32_t in = x.inside(y);
+        if (!in) return;
+#pragma unroll
+        for (int f = 0; f < S::F; ++f) {
+            if (!((in >> f) & 1)) continue;
+            r.y[f] = ey;
+            ++r.n[f];
+            if (!x.also_face_of(f, y)) p.cplx[ey] = 1;
+        }
+    };
+    auto settle = [&](const AdjFrame<TYPE>& x, int32_t v, int32_t e, const Found& r) {
+#pragma unroll
+        for (int f = 0; f < S::F; ++f) {
+            if (!x.smallest(f, v)) continue;
+            p.nbr[(int64_t)e * S::NF + x.slot(f)] = r.n[f] ? r.y[f] : -1;
+            if (r.n[f] > 1) p.cplx[e] = 1;
+        }
+    };
+    int64_t base = warp * PER;
+    auto row = [&](int64_t b0, int64_t& a, int64_t& n) {
+        const int64_t v = b0 + lane / G;
+        a = n = 0;
+        if (v < p.n_nodes) {
+            a = __ldg(p.ne_rp + v);
+            n = __ldg(p.ne_rp + v + 1) - a;
+        }
+    };
+    int64_t r0, L;
+    row(base, r0, L);
+    for (; base < p.n_nodes; base += step) {
+        const int32_t v = (int32_t)(base + lane / G);
+        const int64_t cur = r0, n = L;
+        const int32_t e = n <= G && gl < n ? __ldg(p.ne_col + cur + gl) : -1;
+        row(base + step, r0, L);  // the next node's row, while this one's elements are on their way
+        AdjFrame<TYPE> x{};
+        const int ok = x.load(p, e, v);
+        const int32_t id = ok ? e : -1;
+        if (__any_sync(0xffffffffu, ok == 2)) {
+            // a repeated node: the elements around this node take the slow path
+            const unsigned m = __ballot_sync(0xffffffffu, ok == 2) >> (lane & ~(G - 1));
+            if ((m & (G == 32 ? 0xffffffffu : (1u << (G & 31)) - 1)) && ok) p.cplx[e] = 1;
+        }
+        Found r{};
+        const int jmax = (int)__reduce_max_sync(0xffffffffu, n <= G && n > 1 ? (unsigned)n : 0u);
+        for (int j = 0; j < jmax; ++j) {
+            const int32_t ey = __shfl_sync(0xffffffffu, id, j, G);
+            int32_t y[S::Q];
+#pragma unroll
+            for (int k = 0; k < S::Q; ++k) y[k] = __shfl_sync(0xffffffffu, x.q[k], j, G);
+            if (ok && ey >= 0 && ey != e) compare(x, v, ey, y, r);
+        }
+        if (ok == 1) settle(x, v, e, r);
+        if (n <= G) continue;
+        for (int64_t i = gl; i < n; i += G) {
+            const int32_t ei = __ldg(p.ne_col + cur + i);
+            AdjFrame<TYPE> xi{};
+            const int oki = xi.load(p, ei, v);
+            if (!oki) continue;
+            if (n > ADJ_LONG) {
+                p.cplx[ei] = 1;
+                continue;
+            }
+            Found ri{};
+            for (int64_t j = 0; j < n; ++j) {
+                const int32_t ey = __ldg(p.ne_col + cur + j);
+                AdjFrame<TYPE> y{};
+                const int oky = y.load(p, ey, v);
+                if (oky == 2) p.cplx[ei] = 1;
+                if (oky && ey != ei) compare(xi, v, ey, y.q, ri);
+            }
+            if (oki == 1) settle(xi, v, ei, ri);
+        }
+    }
+}
+
+// The slots of element e, ascending (unsigned: empty ones last).
+template <int NF>
+__device__ __forceinline__ void sorted_slots(const AdjParams& p, int64_t e, uint32_t (&s)[NF]) {
+    if constexpr (NF == 4) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(p.nbr) + e);
+        s[0] = a.x; s[1] = a.y; s[2] = a.z; s[3] = a.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < NF; ++i) s[i] = (uint32_t)__ldg(p.nbr + e * NF + i);
+    }
+    // odd-even transposition: NF rounds
+#pragma unroll
+    for (int r = 0; r < NF; ++r)
+#pragma unroll
+        for (int i = r & 1; i + 1 < NF; i += 2) {
+            const uint32_t x = s[i], y = s[i + 1];
+            s[i] = min(x, y);
+            s[i + 1] = max(x, y);
+        }
+}
+
+// NF: slots per element (0: no slots, every element merges its node rows).
+template <int NF>
 __global__ void __launch_bounds__(ADJ_THREADS) k_adj_count(AdjParams p) {
     for (int64_t e = (int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x; e < p.n_elems;
          e += (int64_t)gridDim.x * ADJ_THREADS) {
         uint32_t c = 0;
-        for_each_neighbour(p, e, [&](int32_t) { ++c; });
+        bool slow = true;
+        if constexpr (NF > 0) {
+            slow = p.cplx[e];
+            if (!slow) {
+                int32_t nd[8];
+                const int t = load_element(p, e, nd);
+                if (t >= 0) {  // (an invalid element is in no node's row: its slots were never written)
+                    uint32_t s[NF];
+                    sorted_slots<NF>(p, e, s);
+#pragma unroll
+                    for (int i = 0; i < NF; ++i) c += s[i] != EMPTY && (i == 0 || s[i] != s[i - 1]);
+                }
+            }
+        }
+        if (slow) for_each_neighbour(p, e, [&](int32_t) { ++c; });
         p.cnt[e] = c;
     }
 }
@@ -155,28 +444,89 @@ __global__ void __launch_bounds__(ADJ_SCAN_THREADS) k_adj_scan(AdjParams p) {
     }
 }
 
+template <int NF>
 __global__ void __launch_bounds__(ADJ_THREADS) k_adj_write(AdjParams p) {
-    for (int64_t e = (int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x; e < p.n_elems;
-         e += (int64_t)gridDim.x * ADJ_THREADS) {
-        const int64_t a = p.rp[e], n = p.rp[e + 1] - a;
-        if (a + n > p.cap) continue;
-        int32_t* row = p.col + a;
-        int64_t k = 0;
-        for_each_neighbour(p, e, [&](int32_t f) {
-            if (k < n) row[k] = f;
-            ++k;
-        });
+    // the rows of a block's elements follow one another: put together in
+    // shared memory and written as one run
+    __shared__ uint32_t rows[NF > 0 ? ADJ_THREADS * NF : 1];
+    for (int64_t e0 = (int64_t)blockIdx.x * ADJ_THREADS; e0 < p.n_elems; e0 += (int64_t)gridDim.x * ADJ_THREADS) {
+        const int64_t e = e0 + threadIdx.x;
+        const int64_t a = e < p.n_elems ? p.rp[e] : 0, n = e < p.n_elems ? p.rp[e + 1] - a : 0;
+        bool slow = n > 0;
+        if constexpr (NF > 0) {
+            slow = n > 0 && p.cplx[e];
+            if (!__syncthreads_or(slow)) {
+                const int64_t a0 = p.rp[e0], a1 = p.rp[min(e0 + ADJ_THREADS, p.n_elems)];
+                if (n > 0) {
+                    uint32_t s[NF];
+                    sorted_slots<NF>(p, e, s);
+                    uint32_t* d = rows + (a - a0);
+#pragma unroll
+                    for (int i = 0; i < NF; ++i)
+                        if (s[i] != EMPTY && (i == 0 || s[i] != s[i - 1])) *d++ = s[i];
+                }
+                __syncthreads();
+                if (a1 <= p.cap)
+                    for (int64_t i = threadIdx.x; i < a1 - a0; i += ADJ_THREADS) p.col[a0 + i] = (int32_t)rows[i];
+                __syncthreads();
+                continue;
+            }
+            if (n > 0 && !slow && a + n <= p.cap) {
+                uint32_t s[NF];
+                sorted_slots<NF>(p, e, s);
+                int32_t* d = p.col + a;
+#pragma unroll
+                for (int i = 0; i < NF; ++i)
+                    if (s[i] != EMPTY && (i == 0 || s[i] != s[i - 1])) *d++ = (int32_t)s[i];
+            }
+        }
+        if (slow && a + n <= p.cap) {
+            int32_t* row = p.col + a;
+            int64_t k = 0;
+            for_each_neighbour(p, e, [&](int32_t f) {
+                if (k < n) row[k] = f;
+                ++k;
+            });
+        }
     }
+}
+
+template <int NF>
+void count_scan_write(const AdjParams& p, int grid, cudaStream_t s) {
+    k_adj_count<NF><<<grid, ADJ_THREADS, 0, s>>>(p);
+    const unsigned tiles = (unsigned)((p.n_elems + ADJ_SCAN_THREADS - 1) / ADJ_SCAN_THREADS);
+    k_adj_scan<<<tiles, ADJ_SCAN_THREADS, 0, s>>>(p);
+    k_adj_write<NF><<<grid, ADJ_THREADS, 0, s>>>(p);
+}
+
+template <int TYPE>
+void match_and_write(const AdjParams& p, int grid, int sms, cudaStream_t s) {
+    constexpr int NODES = ADJ_THREADS / AdjShape<TYPE>::G;  // nodes of a CTA at a time
+    const int64_t blocks = (p.n_nodes + NODES - 1) / NODES;
+    k_adj_match<TYPE><<<(unsigned)(blocks < (int64_t)sms * 16 ? blocks : (int64_t)sms * 16), ADJ_THREADS, 0, s>>>(p);
+    count_scan_write<AdjShape<TYPE>::NF>(p, grid, s);
 }
 
 }  // namespace
 
-cudaError_t launch_adjacency(const AdjParams& p, int grid, cudaStream_t s) {
+// Slots per element of the matching pass; 0: a mixed mesh, whose elements all
+// merge their node rows.
+int adjacency_slots(int type) {
+    return type == NN_TRI ? 3 : (type == NN_QUAD || type == NN_TET ? 4 : (type == NN_HEX ? 6 : 0));
+}
+
+cudaError_t launch_adjacency(const AdjParams& p, int grid, int sms, cudaStream_t s) {
     if (p.n_elems <= 0) return cudaSuccess;
-    k_adj_count<<<grid, ADJ_THREADS, 0, s>>>(p);
-    const unsigned tiles = (unsigned)((p.n_elems + ADJ_SCAN_THREADS - 1) / ADJ_SCAN_THREADS);
-    k_adj_scan<<<tiles, ADJ_SCAN_THREADS, 0, s>>>(p);
-    k_adj_write<<<grid, ADJ_THREADS, 0, s>>>(p);
+    if (!p.nbr) {
+        count_scan_write<0>(p, grid, s);
+        return cudaGetLastError();
+    }
+    switch (p.type) {
+        case NN_TRI: match_and_write<NN_TRI>(p, grid, sms, s); break;
+        case NN_QUAD: match_and_write<NN_QUAD>(p, grid, sms, s); break;
+        case NN_TET: match_and_write<NN_TET>(p, grid, sms, s); break;
+        default: match_and_write<NN_HEX>(p, grid, sms, s); break;
+    }
     return cudaGetLastError();
 }
 

@@ -799,12 +799,26 @@ nn_status nn_plan_info(nn_handle* h, const nn_mesh* mesh, int want, int64_t* inf
     return NN_OK;
 }
 
+namespace {
+
+// Workspace of the counts and the scan, which every call needs, and of the
+// slots and flags of the matching pass.
+size_t adjacency_merge_bytes(size_t T) {
+    return align_up(T * 4) + align_up((adjacency_scan_tiles((int64_t)T) + 1) * 8) + ALIGN;
+}
+size_t adjacency_match_bytes(int type, size_t T) {
+    const size_t slots = (size_t)adjacency_slots(type);
+    return slots ? align_up(T * slots * 4) + align_up(T) : 0;
+}
+
+}  // namespace
+
 nn_status nn_element_neighbors_query(nn_handle* h, const nn_mesh* mesh, size_t* ws_bytes, int64_t* col_cap) {
     if (!h) return NN_ERR_ARG;
     nn_status st = check_mesh(mesh);
     if (st != NN_OK) return st;
     const size_t T = (size_t)mesh->n_elems;
-    if (ws_bytes) *ws_bytes = align_up(T * 4) + align_up((adjacency_scan_tiles((int64_t)T) + 1) * 8) + ALIGN;
+    if (ws_bytes) *ws_bytes = adjacency_merge_bytes(T) + adjacency_match_bytes(mesh->type, T);
     // faces per element (6 at most) times two
     if (col_cap) *col_cap = (int64_t)T * (mesh->type == NN_TRI ? 6 : mesh->type == NN_HEX || mesh->type == NN_MIXED ? 12 : 8);
     return NN_OK;
@@ -817,8 +831,7 @@ nn_status nn_element_neighbors(nn_handle* h, const nn_mesh* mesh, const nn_csr* 
     if (st != NN_OK) return st;
     if (out->col_capacity < 0 || (out->col_capacity > 0 && !out->col)) return NN_ERR_ARG;
     if (mesh->n_conn > 0 && !node_elems->col) return NN_ERR_ARG;
-    size_t need = 0;
-    nn_element_neighbors_query(h, mesh, &need, nullptr);
+    const size_t need = adjacency_merge_bytes((size_t)mesh->n_elems);
     if (ws_bytes < need || !ws || (reinterpret_cast<uintptr_t>(ws) & (ALIGN - 1))) return NN_ERR_WORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     uint8_t* w = static_cast<uint8_t*>(ws);
@@ -844,8 +857,16 @@ nn_status nn_element_neighbors(nn_handle* h, const nn_mesh* mesh, const nn_csr* 
     p.col = out->col;
     p.cap = out->col_capacity;
     p.status = d_status;
+    // a workspace without room for the slots still serves: every element then
+    // merges its node rows
+    const size_t match = adjacency_match_bytes(mesh->type, T);
+    if (match && ws_bytes >= need + match) {
+        p.nbr = reinterpret_cast<int32_t*>(w + need);
+        p.cplx = w + need + match - align_up(T);
+        if (cudaMemsetAsync(p.cplx, 0, T, s) != cudaSuccess) return NN_ERR_CUDA;
+    }
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sms * 8, ((int64_t)T + 255) / 256));
-    return launch_adjacency(p, grid, s) == cudaSuccess ? NN_OK : NN_ERR_CUDA;
+    return launch_adjacency(p, grid, h->sms, s) == cudaSuccess ? NN_OK : NN_ERR_CUDA;
 }
 
 nn_status nn_set_tuning(nn_handle* h, const nn_tuning* t) {

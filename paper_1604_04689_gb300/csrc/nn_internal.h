@@ -183,6 +183,8 @@ struct AdjParams {
     const int64_t* ne_rp;    // node -> element CSR
     const int32_t* ne_col;
     uint32_t* cnt;           // [n_elems] neighbours per element
+    int32_t* nbr;            // [n_elems][adjacency_slots] the element across each face, -1: none (nullptr: merge only)
+    uint8_t* cplx;           // [n_elems] 1: slots do not tell all, merge the node rows (with nbr)
     uint64_t* lb_state;      // lookback words, one per tile of elements
     uint32_t* ticket;
     int64_t* rp; int32_t* col; int64_t cap;
@@ -190,7 +192,8 @@ struct AdjParams {
 };
 
 // launchers (return the CUDA error of the launch)
-cudaError_t launch_adjacency(const AdjParams& p, int grid, cudaStream_t s);
+cudaError_t launch_adjacency(const AdjParams& p, int grid, int sms, cudaStream_t s);
+int adjacency_slots(int type);
 size_t adjacency_scan_tiles(int64_t n_elems);
 cudaError_t launch_node_compact(const CompactParams& p, int copy_grid, cudaStream_t s);
 // chunked builds: base[0] += estart[B], base[1] += nstart[B] (either may be nullptr)
