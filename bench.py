@@ -1036,7 +1036,8 @@ def launches_per_build(plan, want="both"):
 
 # the sources that compile the single-mesh build's kernels and their launch
 # plan: traffic counters taken on other sources no longer describe them
-MEASURED_SOURCES = ("nn_api.cu", "nn_bucket.cu", "nn_bulk.cuh", "nn_compact.cu", "nn_device.cuh", "nn_emit.cu",
+MEASURED_SOURCES = ("nn_api.cu", "nn_bucket.cu", "nn_bucket.cuh", "nn_bucket16.cu",
+                    "nn_bucket32.cu", "nn_bulk.cuh", "nn_compact.cu", "nn_device.cuh", "nn_emit.cu",
                     "nn_internal.h")
 
 

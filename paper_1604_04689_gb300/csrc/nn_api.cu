@@ -62,16 +62,15 @@ struct Plan {
     int G_part = 1;
     int G_fine = 1;
     size_t emit_smem = 0;
-    size_t off_estart = 0, off_nfc = 0, off_ntmp = 0, off_ubk = 0, off_nloc = 0, off_nstart = 0, off_lb_ns = 0;
+    size_t off_estart = 0, off_nfc = 0, off_ntmp = 0, off_grp = 0, off_nloc = 0, off_nstart = 0, off_lb_ns = 0;
     size_t off_hist = 0, off_bstart = 0, off_gcur = 0, off_gcur_c = 0, off_rec_tmp = 0, off_rec = 0, off_lb_off = 0,
            off_ctrl = 0, off_spill = 0, zero_begin = 0, zero_end = 0;
     size_t ws_min = 0, ws_rec = 0;
     int bucket_grid = 0;
     int bucket_threads = 256;
-    int wide = 0;
-    int rec_smem = 1;
+    int imax = 32, slots = 8, list_cap = 32;  // bucket pass: variant, places per node, listed records
+    int groups = 1;                           // groups of 32 nodes per bucket
     size_t bucket_smem = 0;
-    uint32_t area_words = 0;
 };
 
 nn_status check_mesh(const nn_mesh* m) {
@@ -107,73 +106,43 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     p.n_conn = records;
     p.k = (m->type == NN_TRI || m->type == NN_QUAD) ? 2 : 3;
 
-    // bucket kernel shape.  Every node goes to one lane, which holds up to
-    // 16 (or, "wide", 32) records and a 16 (32) slot neighbour table;
-    // meshes whose nodes have more than ten incidences on average (tets,
-    // mixed) take the wide form.  256-thread CTAs, two per SM.  A bucket's
-    // records are copied into the CTA's shared memory beside each record's
-    // slot, its record groups, element rows and neighbour rows; the bucket
-    // width is as many nodes as fit with room to spare for buckets of higher
-    // than average record counts.
+    // bucket kernel shape (nn_bucket.cuh).  Slots per node: 8 for meshes of up
+    // to 8 incidences per node (triangles, quads, hexes), 16 up to 10, else
+    // about the mean and at least 24 (a node with more uses the bucket's list,
+    // which costs its warp a second sort: mixed hex and tet meshes, 13 on
+    // average, often have 20); the slots also pick the variant by its register
+    // arrays.  A bucket has as many nodes as the CTA has lanes: 256, or 128
+    // where a node's columns are so long that two CTAs of 256 do not fit.
     const double inc = p.N > 0 ? (double)p.n_conn / (double)p.N : 0.0;
-    p.wide = inc > 10.0 ? 1 : 0;
-    const int ucap = p.wide ? 24 : 12;  // distinct neighbours a lane's table takes
-    p.bucket_threads = h->tuning.bucket_threads ? h->tuning.bucket_threads : 256;
-    const int bcps = h->tuning.bucket_ctas_per_sm ? h->tuning.bucket_ctas_per_sm : (p.bucket_threads == 128 ? 4 : 2);
-    size_t bsmem = std::min(h->bucket_smem, h->smem_per_sm / (size_t)bcps - 2048);
-    // distinct neighbours per node: half the candidates, at most two thirds
-    // of what a lane's table takes (a Kuhn tet grid has 14 for 72 candidates)
-    const double U = (want & NN_WANT_NODES) ? std::min(p.k * inc / 2.0, ucap * 2.0 / 3.0) : 0.0;
-    // record width of a bucket shift s (the fine-digit field of a two-level
-    // partition included, at most 12 bits)
-    const int eb_ = bits_for(p.T > 0 ? (uint64_t)(p.T - 1) : 0), nb_ = bits_for((uint64_t)m->n_nodes);
-    auto rb_of = [&](int s) {
-        const int bits = s + ((want & NN_WANT_ELEMS) ? 1 + eb_ : 0) + ((want & NN_WANT_NODES) ? p.k * nb_ : 0);
-        int cs_ = 0;
-        while ((((p.N + (1ll << s) - 1) >> s) + (1ll << cs_) - 1) >> cs_ > 256) ++cs_;
-        return bits + cs_ <= 64 ? 8 : 16;
-    };
-    // shared memory of a bucket of 2^s nodes with 15 % more records than
-    // average: the records themselves (when copied in), a slot and a group
-    // entry per record, element rows, neighbour rows
-    bool rec_smem = true;
-    auto bucket_bytes = [&](int s) {
-        const double n = (double)(1 << s) * 1.15;
-        return n * (inc * ((rec_smem ? rb_of(s) : 0) + 8.0) + 4.0 * (rec_smem ? std::max(U, inc) : U)) + 64.0;
-    };
-    // (many buckets are fine: the histogram pass counts them in chunks that
-    // fit its shared memory; the hard cap below only bounds workspace tables)
-    const int64_t B_lim = (int64_t)1 << 20;
-    auto fixed_of = [&](int s) { return bucket_fixed_bytes(s, p.bucket_threads, p.wide); };
-    auto widest = [&]() {
-        for (int s = SB_MAX; s >= SB_MIN; --s) {
-            if (((p.N + (1ll << s) - 1) >> s) > B_lim) break;
-            const double area = (double)bsmem - (double)fixed_of(s);
-            if (area > 0 && bucket_bytes(s) <= area) return s;
-        }
-        return -1;
-    };
-    // records in shared memory unless that leaves a bucket fewer nodes than
-    // the CTA has lanes
-    int sb = widest();
-    if (sb >= 0 && (32 << (sb - 5)) < p.bucket_threads && sb < SB_MAX) {
-        rec_smem = false;
-        const int s2 = widest();
-        if (s2 > sb) sb = s2;
-        else rec_smem = true;
+    p.imax = inc <= 8.0 ? 8 : (inc <= 10.0 ? 16 : 32);
+    const int want_slots = p.imax < 32 ? p.imax : std::min(32, std::max(24, 4 * (int)std::ceil(inc / 4.0)));
+    auto nbk = [&](int s) { return (p.N + (1ll << s) - 1) >> s; };
+    auto list_of = [&](int s) { return (int)std::max(32.0, std::min(512.0, std::ceil((double)(1 << s) * inc / 12.0 / 16.0) * 16.0)); };
+    auto need = [&](int s, int slots) { return bucket_smem_bytes(s, want, p.k, slots, 16, list_of(s)); };
+    p.bucket_threads = h->tuning.bucket_threads ? h->tuning.bucket_threads
+                       : (need(8, want_slots) <= h->smem_per_sm / 2 - 2048 ? 256 : 128);
+    const int64_t B_max = (int64_t)1 << 20;  // (bounds the workspace tables)
+    int sb = p.bucket_threads == 128 ? 7 : 8;
+    if (h->tuning.bucket_ctas_per_sm) {  // the widest bucket that leaves room for that many CTAs
+        const size_t budget = std::min(h->bucket_smem, h->smem_per_sm / (size_t)h->tuning.bucket_ctas_per_sm - 2048);
+        sb = SB_MAX;
+        while (sb > SB_MIN && need(sb, want_slots) > budget) --sb;
+    } else {
+        // a small mesh: buckets for every SM, as long as one partition pass (256 buckets) does
+        while (sb > 5 && nbk(sb) < 2 * (int64_t)h->sms && nbk(sb - 1) <= 256) --sb;
     }
-    p.rec_smem = rec_smem ? 1 : 0;
-    if (sb < 0) sb = SB_MIN;
     if (h->tuning.sb >= SB_MIN && h->tuning.sb <= SB_MAX) sb = h->tuning.sb;
     if (h->sb_override >= SB_MIN && h->sb_override <= SB_MAX) sb = h->sb_override;
-    const size_t min_area = 1024 * 4;
-    while (fixed_of(sb) + min_area > bsmem && bsmem < h->bucket_smem) bsmem = h->bucket_smem;
-    p.bucket_smem = bsmem;
-    while (sb > SB_MIN && fixed_of(sb) + min_area > p.bucket_smem) --sb;
-    const int64_t B_max = B_lim;
-    auto nbk = [&](int s) { return (p.N + (1ll << s) - 1) >> s; };
+    // wider buckets than shared memory holds (a tuning, a test): fewer slots,
+    // then fewer nodes
+    constexpr int SLOTS_MIN = 4;
+    while (sb > SB_MIN && need(sb, SLOTS_MIN) > h->bucket_smem) --sb;
     while (nbk(sb) > B_max && sb < SB_MAX) ++sb;
-    if (nbk(sb) > B_max || fixed_of(sb) + min_area > p.bucket_smem) return NN_ERR_ARG;
+    if (nbk(sb) > B_max || need(sb, SLOTS_MIN) > h->bucket_smem) return NN_ERR_ARG;
+    p.slots = SLOTS_MIN;
+    while (p.slots < want_slots && need(sb, p.slots + 1) <= h->bucket_smem) ++p.slots;
+    p.list_cap = list_of(sb);
+    p.groups = sb < 5 ? 1 : 1 << (sb - 5);
     p.B = nbk(sb);
 
     RecFmt& f = p.fmt;
@@ -213,21 +182,23 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
         p.G_part = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sms * 4, (n_units + 511) / 512));
     p.G_fine = h->sms;  // the fine pass sizes its grid by its occupancy
 
-    p.area_words = (uint32_t)((p.bucket_smem - fixed_of(sb)) / 4);
+    p.bucket_smem = bucket_smem_bytes(sb, want, p.k, p.slots, f.rb, p.list_cap);
     int per_sm = 1;
-    if (h->offline || bucket_occupancy(&per_sm, p.bucket_threads, p.wide, p.bucket_smem) != cudaSuccess || per_sm < 1)
+    if (h->offline || bucket_occupancy(&per_sm, p.bucket_threads, p.imax, p.bucket_smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     p.bucket_grid = (int)std::min<int64_t>(p.B, (int64_t)h->sms * per_sm);
 
     // workspace layout
     size_t o = 0;
-    p.off_hist = o; o = align_up(o + (size_t)p.G * p.B * 4);
     p.off_bstart = o; o = align_up(o + ((size_t)p.B + 1) * 4);
     p.off_estart = o; o = align_up(o + ((want & NN_WANT_ELEMS) ? ((size_t)p.B + 1) * 4 : 0));
     p.off_gcur = o; o = align_up(o + (size_t)p.B * 4);
     p.off_gcur_c = o; o = align_up(o + 256 * 4);
+    // the histogram rows are dead once the offsets are known: they share the records' place
+    p.off_hist = o;
+    const size_t hist_end = align_up(o + (size_t)p.G * p.B * 4);
     p.off_rec_tmp = o; o = align_up(o + (f.cshift > 0 ? (size_t)p.n_conn * f.rb : 0));
-    p.off_rec = o; o = align_up(o + (size_t)p.n_conn * f.rb);
+    p.off_rec = o; o = std::max(hist_end, align_up(o + (size_t)p.n_conn * f.rb));
     // node rows in scratch (at most k per record), per-node offsets within
     // their bucket, bucket totals and their scan
     const bool wn = want & NN_WANT_NODES;
@@ -237,25 +208,24 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     } else {
         p.off_ntmp = o; o = align_up(o + ntmp_bytes);
     }
-    p.off_ubk = o; o = align_up(o + (wn ? (size_t)p.B * 4 : 0));
+    const size_t ngrp = (size_t)p.B * p.groups;
+    p.off_grp = o; o = align_up(o + (wn ? ngrp * 8 : 0));
     p.off_nloc = o; o = align_up(o + (wn ? ((size_t)p.B << sb) * 4 : 0));
-    p.off_nstart = o; o = align_up(o + (wn ? ((size_t)p.B + 1) * 8 : 0));
+    p.off_nstart = o; o = align_up(o + (wn ? (ngrp + 1) * 8 : 0));
     p.zero_begin = o;
     p.off_nfc = o; o = align_up(o + ((want & NN_WANT_ELEMS) ? (size_t)p.B * 4 : 0));
     p.off_lb_off = o; o = align_up(o + (size_t)((p.B + OFFSETS_THREADS - 1) / OFFSETS_THREADS) * 8 + 8);
-    p.off_lb_ns = o; o = align_up(o + (wn ? (size_t)((p.B + 127) / 128) * 8 + 8 : 0));
+    p.off_lb_ns = o; o = align_up(o + (wn ? (ngrp + NODE_SCAN_TILE - 1) / NODE_SCAN_TILE * 8 + 8 : 0));
     p.off_ctrl = o; o = align_up(o + 64);
     p.zero_end = o;
     p.off_spill = o;
     p.ws_min = o;
-    // spill area: buckets larger than the bucket pass's shared memory keep
-    // their record groups and rows there (16 MB and 8 bytes per record covers
-    // the odd oversized bucket, a node of very high valence included); a
-    // plan whose typical bucket does not fit (a tuning that widens the
-    // buckets) gets room for all of them
+    // spill area: buckets built by a whole CTA group their record indices and
+    // sort long rows there (16 MB and 8 bytes per record covers the odd node
+    // of very high valence); a plan whose typical bucket has too few slots (a
+    // tuning that widens the buckets) gets room for all of them
     size_t spill = ((size_t)16 << 20) + (size_t)p.n_conn * 8;
-    if (bucket_bytes(sb) > (double)p.area_words * 4.0)
-        spill += (size_t)p.n_conn * (8 + 4 * (size_t)p.k) + (size_t)p.B * 64;
+    if (p.slots < want_slots) spill += (size_t)p.n_conn * (8 + 4 * (size_t)p.k) + (size_t)p.B * 64;
     p.ws_rec = o + spill;
 
     *P = p;
@@ -398,16 +368,16 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     }
     bp.base = base;
     bp.status = d_status;
-    bp.area_words = p.area_words;
-    bp.wide = p.wide;
-    bp.rec_smem = p.rec_smem;
+    bp.imax = p.imax;
+    bp.slots = p.slots;
+    bp.list_cap = p.list_cap;
     bp.ntmp = reinterpret_cast<uint32_t*>(w + p.off_ntmp);
-    bp.ubk = reinterpret_cast<uint32_t*>(w + p.off_ubk);
+    bp.grp = reinterpret_cast<uint2*>(w + p.off_grp);
     bp.nloc = reinterpret_cast<uint32_t*>(w + p.off_nloc);
     bp.rec_count = (uint64_t)p.n_conn;
     bp.ntmp_words = (want & NN_WANT_NODES) ? (uint64_t)p.k * p.n_conn + 4 : 0;
     bp.nloc_words = (want & NN_WANT_NODES) ? (uint64_t)p.B << p.fmt.sb : 0;
-    bp.ubk_words = (want & NN_WANT_NODES) ? (uint64_t)p.B : 0;
+    bp.ngrp = (want & NN_WANT_NODES) ? (uint64_t)p.B * p.groups : 0;
 
     mark(1);
     if (launch_hist(ep, p.emit_smem, s) != cudaSuccess) return NN_ERR_CUDA;
@@ -429,13 +399,12 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     if (want & NN_WANT_NODES) {
         CompactParams cp{};
         cp.n_buckets = p.B;
-        cp.n_buckets_cap = p.B;
+        cp.n_groups_cap = p.B * p.groups;
         cp.sb = p.fmt.sb;
         cp.k = p.k;
         cp.n_nodes = p.N;
         cp.base = base;
-        cp.bstart = bp.bstart;
-        cp.ubk = bp.ubk;
+        cp.grp = bp.grp;
         cp.nloc = bp.nloc;
         cp.ntmp = bp.ntmp;
         cp.nstart = reinterpret_cast<uint64_t*>(w + p.off_nstart);
@@ -447,7 +416,7 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
         cp.status = d_status;
         cp.ntmp_words = bp.ntmp_words;
         cp.nloc_words = bp.nloc_words;
-        if (launch_node_compact(cp, (int)std::min<int64_t>(p.B, (int64_t)h->sms * 8), s) != cudaSuccess)
+        if (launch_node_compact(cp, (int)std::min<int64_t>((cp.n_groups_cap + 7) / 8, (int64_t)h->sms * 8), s) != cudaSuccess)
             return NN_ERR_CUDA;
     }
     mark(7);
@@ -456,14 +425,15 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
 
 // --------------------------------------------------------------- batches
 
+constexpr int BATCH_SLOTS = 24, BATCH_LIST = 256;
+
 struct BatchPlan {
-    int sb = 7;
+    int sb = 7, groups = 4;
     int64_t B_cap = 0;
     size_t hdr_bytes = 0, meshes_off = 0, elem_off_off = 0, bucket_off_off = 0, table_bytes = 0;
     size_t off_bcount = 0, off_bstart = 0, off_gcur = 0, off_rec = 0, off_lb_off = 0, off_ctrl = 0, off_spill = 0, ws_min = 0, ws_rec = 0, off_nfc = 0,
-           off_estart = 0, off_ntmp = 0, off_ubk = 0, off_nloc = 0, off_nstart = 0, off_lb_ns = 0;
+           off_estart = 0, off_ntmp = 0, off_grp = 0, off_nloc = 0, off_nstart = 0, off_lb_ns = 0;
     size_t bucket_smem = 0;
-    uint32_t area_words = 0;
     int bucket_grid = 0, emit_grid = 0, bucket_threads = 128;
     int64_t tiles_cap = 0;
 };
@@ -476,23 +446,21 @@ nn_status batch_plan(const nn_handle* h, const nn_batch_caps* c, BatchPlan* out)
     BatchPlan p;
     p.sb = c->sb ? c->sb : 7;
     if (p.sb < SB_MIN || p.sb > SB_MAX) return NN_ERR_ARG;
-    p.B_cap = (c->max_nodes >> p.sb) + c->max_meshes + 1;
     p.hdr_bytes = align_up(sizeof(BatchHeader));
     p.meshes_off = p.hdr_bytes;
     p.elem_off_off = p.meshes_off + align_up((size_t)c->max_meshes * sizeof(BatchMesh));
     p.bucket_off_off = p.elem_off_off + align_up(((size_t)c->max_meshes + 1) * 8);
     p.table_bytes = p.bucket_off_off + align_up(((size_t)c->max_meshes + 1) * 8);
-    // bucket kernel: wide lanes (a batch may hold any element type), 256
-    // threads, two CTAs per SM, so that a bucket's records (copied into
-    // shared memory) fit beside its tables
-    p.bucket_threads = 256;
-    const size_t fixed = bucket_fixed_bytes(p.sb, p.bucket_threads, 1);
-    p.bucket_smem = std::min(h->bucket_smem, h->smem_per_sm / 2 - 2048);
-    if (fixed + 8192 * 4 > p.bucket_smem) p.bucket_smem = h->bucket_smem;
-    if (fixed + 4096 * 4 > p.bucket_smem) return NN_ERR_ARG;
-    p.area_words = (uint32_t)((p.bucket_smem - fixed) / 4);
+    // bucket kernel: the 24 slots of a tet mesh (a batch may hold any element
+    // type), 128 threads for buckets of 128 nodes
+    p.bucket_threads = 128;
+    while (p.sb > SB_MIN && bucket_smem_bytes(p.sb, c->want, 3, BATCH_SLOTS, 16, BATCH_LIST) > h->bucket_smem) --p.sb;
+    p.bucket_smem = bucket_smem_bytes(p.sb, c->want, 3, BATCH_SLOTS, 16, BATCH_LIST);
+    if (p.bucket_smem > h->bucket_smem) return NN_ERR_ARG;
+    p.groups = p.sb < 5 ? 1 : 1 << (p.sb - 5);
+    p.B_cap = (c->max_nodes >> p.sb) + c->max_meshes + 1;
     int per_sm = 1;
-    if (bucket_occupancy(&per_sm, p.bucket_threads, 1, p.bucket_smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (bucket_occupancy(&per_sm, p.bucket_threads, 32, p.bucket_smem) != cudaSuccess || per_sm < 1) per_sm = 1;
     p.bucket_grid = h->sms * per_sm;
     size_t o = p.table_bytes;
     p.off_bcount = o; o = align_up(o + (size_t)p.B_cap * 4);
@@ -503,10 +471,11 @@ nn_status batch_plan(const nn_handle* h, const nn_batch_caps* c, BatchPlan* out)
     p.off_rec = o; o = align_up(o + (size_t)c->max_conn * 16);
     const bool wn = c->want & NN_WANT_NODES;
     p.off_ntmp = o; o = align_up(o + (wn ? (size_t)3 * c->max_conn * 4 + 16 : 0));
-    p.off_ubk = o; o = align_up(o + (wn ? (size_t)p.B_cap * 4 : 0));
+    const size_t ngrp = (size_t)p.B_cap * p.groups;
+    p.off_grp = o; o = align_up(o + (wn ? ngrp * 8 : 0));
     p.off_nloc = o; o = align_up(o + (wn ? ((size_t)p.B_cap << p.sb) * 4 : 0));
-    p.off_nstart = o; o = align_up(o + (wn ? ((size_t)p.B_cap + 1) * 8 : 0));
-    p.off_lb_ns = o; o = align_up(o + (wn ? (size_t)((p.B_cap + 127) / 128) * 8 + 8 : 0));
+    p.off_nstart = o; o = align_up(o + (wn ? (ngrp + 1) * 8 : 0));
+    p.off_lb_ns = o; o = align_up(o + (wn ? (ngrp + NODE_SCAN_TILE - 1) / NODE_SCAN_TILE * 8 + 8 : 0));
     p.tiles_cap = (p.B_cap + OFFSETS_THREADS - 1) / OFFSETS_THREADS;
     p.off_lb_off = o; o = align_up(o + ((size_t)p.tiles_cap + 1) * 8);
     p.off_ctrl = o; o = align_up(o + 64);
@@ -643,26 +612,25 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     kp.spill = reinterpret_cast<uint32_t*>(w + bp.off_spill);
     const size_t spill_bytes = ws_bytes > bp.off_spill ? ws_bytes - bp.off_spill : 0;
     kp.spill_words = spill_bytes / 4;
-    kp.area_words = bp.area_words;
     kp.batch = bt;
     kp.batch_err = reinterpret_cast<const int32_t*>(ctrl + 8);
     kp.fmt.rb = 16;
     kp.fmt.k = 3;
-    kp.wide = 1;
-    kp.rec_smem = 1;
+    kp.imax = 32;
+    kp.slots = BATCH_SLOTS;
+    kp.list_cap = BATCH_LIST;
     kp.ntmp = reinterpret_cast<uint32_t*>(w + bp.off_ntmp);
-    kp.ubk = reinterpret_cast<uint32_t*>(w + bp.off_ubk);
+    kp.grp = reinterpret_cast<uint2*>(w + bp.off_grp);
     kp.nloc = reinterpret_cast<uint32_t*>(w + bp.off_nloc);
     kp.rec_count = (uint64_t)c->max_conn;
     kp.ntmp_words = (c->want & NN_WANT_NODES) ? 3 * (uint64_t)c->max_conn + 4 : 0;
     kp.nloc_words = (c->want & NN_WANT_NODES) ? (uint64_t)bp.B_cap << bp.sb : 0;
-    kp.ubk_words = (c->want & NN_WANT_NODES) ? (uint64_t)bp.B_cap : 0;
+    kp.ngrp = (c->want & NN_WANT_NODES) ? (uint64_t)bp.B_cap * bp.groups : 0;
     if (launch_bucket(kp, bp.bucket_grid, bp.bucket_threads, bp.bucket_smem, s) != cudaSuccess) return NN_ERR_CUDA;
     if (c->want & NN_WANT_NODES) {
         CompactParams cp{};
-        cp.n_buckets_cap = bp.B_cap;
-        cp.bstart = kp.bstart;
-        cp.ubk = kp.ubk;
+        cp.n_groups_cap = bp.B_cap * bp.groups;
+        cp.grp = kp.grp;
         cp.nloc = kp.nloc;
         cp.ntmp = kp.ntmp;
         cp.nstart = reinterpret_cast<uint64_t*>(w + bp.off_nstart);
@@ -1074,9 +1042,10 @@ nn_status nn_neighbors_chunked(nn_handle* h, const nn_mesh* mesh, int want, cons
         make_plan_range(h, mesh, want, chunks[c].node_lo, chunks[c].node_hi - chunks[c].node_lo, chunks[c].records, &p);
         if ((st = enqueue(h, mesh, p, nodes, elems, cw, ws_bytes - ALIGN, base, d_status, false, s)) != NN_OK)
             return st;
-        const uint32_t* estart = (want & NN_WANT_ELEMS) ? reinterpret_cast<const uint32_t*>(cw + p.off_estart) : nullptr;
-        const uint64_t* nstart = (want & NN_WANT_NODES) ? reinterpret_cast<const uint64_t*>(cw + p.off_nstart) : nullptr;
-        if (launch_chunk_advance(base, estart, nstart, p.B, s) != cudaSuccess) return NN_ERR_CUDA;
+        // (the chunk's totals end its two scans)
+        const uint32_t* etot = (want & NN_WANT_ELEMS) ? reinterpret_cast<const uint32_t*>(cw + p.off_estart) + p.B : nullptr;
+        const uint64_t* ntot = (want & NN_WANT_NODES) ? reinterpret_cast<const uint64_t*>(cw + p.off_nstart) + p.B * p.groups : nullptr;
+        if (launch_chunk_advance(base, etot, ntot, s) != cudaSuccess) return NN_ERR_CUDA;
     }
     return NN_OK;
 }

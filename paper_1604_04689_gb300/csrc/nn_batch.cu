@@ -103,7 +103,9 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_batch_init(BatchTables bt, ui
     }
     for (int64_t i = i0; i < tiles + 1; i += st) lb_off[i] = 0;
     if (lb_ns)
-        for (int64_t i = i0; i < (B + 127) / 128 + 1; i += st) lb_ns[i] = 0;
+        for (int64_t i = i0, n = B * (bt.hdr->fmt.sb < 5 ? 1 : 1 << (bt.hdr->fmt.sb - 5));
+             i < (n + NODE_SCAN_TILE - 1) / NODE_SCAN_TILE + 1; i += st)
+            lb_ns[i] = 0;
     for (int64_t i = i0; i < 16; i += st) ctrl[i] = 0;
     for (int64_t i = i0; i < n; i += st) {
         const BatchMesh& M = bt.meshes[i];

@@ -115,7 +115,8 @@ struct BatchTables {
 };
 
 // Bucket pass: one CTA per bucket (persistent, buckets taken in order),
-// builds the rows of the bucket's 2^sb nodes and writes both CSRs.
+// builds the rows of the bucket's 2^sb nodes in groups of 32 (or of 2^sb,
+// if fewer).
 struct BucketParams {
     RecFmt fmt;
     int64_t n_nodes;
@@ -130,12 +131,12 @@ struct BucketParams {
     int64_t* rp_n; int32_t* col_n; int64_t cap_n;
     int64_t* rp_e; int32_t* col_e; int64_t cap_e;
     int32_t* status;
-    uint32_t area_words;    // shared-memory words available for record groups and rows
-    uint32_t* ntmp;         // node rows of bucket b at ntmp + k * bstart[b] (k = neighbours per record)
-    uint32_t* ubk;          // [n_buckets] node-row total of each bucket
-    uint32_t* nloc;         // [n_buckets << sb] each node's offset within its bucket's rows
-    int32_t wide;           // 1: 32 records and a 32-slot table per node in registers, 0: 16 and 16
-    int32_t rec_smem;       // 1: copy each bucket's records into shared memory when they fit, 0: read them from L2
+    uint32_t* ntmp;         // node rows of a group of 32 nodes at ntmp + k * its first record (k = neighbours per record)
+    uint2* grp;             // [n_buckets * groups] each group's first record and node-row total
+    uint32_t* nloc;         // [n_buckets << sb] each node's offset within its group's rows
+    int32_t imax;           // 8, 16 or 32: the variant by its register arrays
+    int32_t slots;          // places per node in the shared-memory table (<= imax)
+    int32_t list_cap;       // records beyond their node's slots that a bucket may have
     BatchTables batch;      // batch.hdr != nullptr: format, bucket count and meshes come from the tables
     const int32_t* batch_err;  // batches: status of the shared offsets scan, copied to every mesh
     const int64_t* base;    // chunked builds: {element-CSR, node-CSR} entries of the earlier chunks (else nullptr)
@@ -143,26 +144,26 @@ struct BucketParams {
     uint64_t rec_count;     // records the record array holds
     uint64_t ntmp_words;    // words of ntmp
     uint64_t nloc_words;    // words of nloc
-    uint64_t ubk_words;     // words of ubk
+    uint64_t ngrp;          // entries of grp
 };
 
 constexpr int EMIT_THREADS = 1024;
 constexpr int PART_THREADS = 512;
 constexpr int SORT_THREADS = 256;   // tile-sorted partition passes
 constexpr int OFFSETS_THREADS = 128;
+constexpr int NODE_SCAN_TILE = 512;  // groups of 32 nodes per tile of the node-row placement's scan
 
 // Placement of the node rows the bucket pass left in scratch (nn_compact.cu).
 struct CompactParams {
     int64_t n_buckets;       // single mesh (batches: from the header)
-    int64_t n_buckets_cap;   // grid of the scan (batches: capacity)
+    int64_t n_groups_cap;    // grid of the scan (batches: capacity)
     int sb, k;               // single mesh (batches: from the header; k = 3)
     int64_t n_nodes;
-    const uint32_t* bstart;
-    const uint32_t* ubk;
+    const uint2* grp;        // [n_buckets * groups] first record and node-row total of each group of 32 nodes
     const uint32_t* nloc;
     const uint32_t* ntmp;
-    uint64_t* nstart;        // [n_buckets+1] exclusive scan of ubk (batch-wide)
-    uint64_t* lb_state;      // lookback words, one per tile of buckets
+    uint64_t* nstart;        // [n_buckets * groups + 1] exclusive scan of the totals (batch-wide)
+    uint64_t* lb_state;      // lookback words, one per tile of groups
     uint32_t* ticket;
     int64_t* rp_n; int32_t* col_n; int64_t cap_n;
     int32_t* status;
@@ -196,9 +197,8 @@ cudaError_t launch_adjacency(const AdjParams& p, int grid, int sms, cudaStream_t
 int adjacency_slots(int type);
 size_t adjacency_scan_tiles(int64_t n_elems);
 cudaError_t launch_node_compact(const CompactParams& p, int copy_grid, cudaStream_t s);
-// chunked builds: base[0] += estart[B], base[1] += nstart[B] (either may be nullptr)
-cudaError_t launch_chunk_advance(int64_t* base, const uint32_t* estart, const uint64_t* nstart, int64_t B,
-                                 cudaStream_t s);
+// chunked builds: base[0] += *etot, base[1] += *ntot (either may be nullptr)
+cudaError_t launch_chunk_advance(int64_t* base, const uint32_t* etot, const uint64_t* ntot, cudaStream_t s);
 // incidences per node slab of 2^shift nodes, added to counts[0 .. n_slabs) (n_slabs <= NN_CHUNK_SLABS_MAX)
 cudaError_t launch_slab_count(const EmitParams& p, int shift, int n_slabs, uint32_t* counts, cudaStream_t s);
 cudaError_t launch_hist(const EmitParams& p, size_t smem, cudaStream_t s);
@@ -209,8 +209,9 @@ cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s);
 cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s);
 cudaError_t launch_offsets(const OffsetsParams& p, cudaStream_t s);
 cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
-size_t bucket_fixed_bytes(int sb, int threads, int wide);  // shared memory of the bucket kernel outside its area
-cudaError_t bucket_occupancy(int* blocks, int threads, int wide, size_t smem);
+// dynamic shared memory of the bucket kernel for buckets of 2^sb nodes
+size_t bucket_smem_bytes(int sb, int want, int k, int slots, int rb, int list_cap);
+cudaError_t bucket_occupancy(int* blocks, int threads, int imax, size_t smem);
 cudaError_t launch_batch_emit(const BatchTables& bt, uint32_t* bcount, uint32_t* nfc, uint32_t* gcur, uint8_t* rec,
                               uint64_t* lb_off, uint32_t* ctrl, int grid, int stage, cudaStream_t s,
                               uint64_t* lb_ns = nullptr);
