@@ -87,6 +87,34 @@ nn_status check_mesh(const nn_mesh* m) {
     return NN_OK;
 }
 
+// Record format (see RecFmt) for ids of T elements and N nodes; false when the
+// fields exceed 128 bits.  rb: 16 forces 16-byte records.
+bool record_format(int sb, int want, int k, int64_t T, int64_t N, int cshift, int rb, RecFmt* out) {
+    const bool we = want & NN_WANT_ELEMS, wn = want & NN_WANT_NODES;
+    RecFmt f{};
+    f.sb = sb;
+    f.want = want;
+    f.k = k;
+    f.cshift = cshift;
+    f.eb = bits_for(T > 0 ? (uint64_t)(T - 1) : 0);
+    f.nb = bits_for((uint64_t)N);  // (an id below N is never all ones)
+    f.emask = (uint32_t)((1ull << f.eb) - 1);
+    f.nmask = (uint32_t)((1ull << f.nb) - 1);
+    f.off_nf = sb + (cshift > 0 ? cshift : 0);
+    const int side = f.off_nf + (we ? 1 : 0);
+    f.off_e = side;
+    f.off_n = side + (we ? f.eb : 0);
+    const int total = f.off_n + (wn ? k * f.nb : 0);
+    if (total > 128) return false;
+    f.rb = rb == 16 || total > 64 ? 16 : 8;
+    f.side_split = we && wn && k == 3;
+    f.sh2 = std::min(31, 32 - f.nb);
+    f.sh3 = std::min(31, 2 * (32 - f.nb));
+    f.sh0 = std::min(31, 3 * (32 - f.nb));
+    *out = f;
+    return true;
+}
+
 // Plan of a build over the nodes [lo, lo + span) of mesh m, which have
 // `records` incidences: the element walk covers the whole mesh, the record
 // arrays and node tables only this range.  Record fields stay sized by the
@@ -145,28 +173,15 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     p.groups = sb < 5 ? 1 : 1 << (sb - 5);
     p.B = nbk(sb);
 
-    RecFmt& f = p.fmt;
-    f.sb = sb;
-    f.want = want;
-    f.k = p.k;
-    f.eb = bits_for(p.T > 0 ? (uint64_t)(p.T - 1) : 0);
-    f.nb = bits_for((uint64_t)m->n_nodes);
-    f.off_nf = sb;
-    f.off_e = sb + 1;
-    f.off_n = (want & NN_WANT_ELEMS) ? sb + 1 + f.eb : sb;
-    int total = (want & NN_WANT_NODES) ? f.off_n + p.k * f.nb : sb + 1 + f.eb;
-    if (total > 128) return NN_ERR_ARG;
     // partition: tile-sorted (one pass for <= 256 buckets, else coarse + fine
     // with the fine digit kept in the record) unless that field does not fit
     int cs = 0;
     while (((p.B + (1ll << cs) - 1) >> cs) > 256) ++cs;
-    f.cshift = -1;
-    f.off_fb = total;
-    if (h->part_mode != 0 && total + cs <= 128 && cs <= 12) {  // <= 4096 buckets per coarse region
-        f.cshift = cs;
-        total += cs;
-    }
-    f.rb = total <= 64 ? 8 : 16;
+    RecFmt& f = p.fmt;
+    const bool sorted = h->part_mode != 0 && cs <= 12;  // <= 4096 buckets per coarse region
+    if (!(sorted && record_format(sb, want, p.k, p.T, m->n_nodes, cs, 0, &f)) &&
+        !record_format(sb, want, p.k, p.T, m->n_nodes, -1, 0, &f))
+        return NN_ERR_ARG;
 
     // element-walk CTAs: one or two per SM, each a fixed slice of elements
     const int unit = p.type == NN_TRI ? 4 : 1;
@@ -539,19 +554,7 @@ nn_status batch_prepare(nn_handle* h, const nn_batch_caps* c, const nn_mesh* mes
     boff[n] = Bk;
     if (E > c->max_elems || C > c->max_conn || Nn > c->max_nodes || Bk > bp.B_cap) return NN_ERR_BUDGET;
     RecFmt f{};
-    f.sb = bp.sb;
-    f.want = c->want;
-    f.k = 3;
-    f.eb = bits_for(maxT > 0 ? (uint64_t)(maxT - 1) : 0);
-    f.nb = bits_for((uint64_t)maxN);
-    f.off_nf = f.sb;
-    f.off_e = f.sb + 1;
-    f.off_n = (c->want & NN_WANT_ELEMS) ? f.sb + 1 + f.eb : f.sb;
-    const int total = (c->want & NN_WANT_NODES) ? f.off_n + 3 * f.nb : f.sb + 1 + f.eb;
-    if (total > 128) return NN_ERR_ARG;
-    f.rb = 16;
-    f.cshift = -1;
-    f.off_fb = total;
+    if (!record_format(bp.sb, c->want, 3, maxT, maxN, -1, 16, &f)) return NN_ERR_ARG;
     hdr->fmt = f;
     hdr->n_meshes = n;
     hdr->n_elems = E;

@@ -140,7 +140,6 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_hist_b(BatchTables bt, uint32
 __global__ void __launch_bounds__(BATCH_THREADS) k_part_b(BatchTables bt, uint32_t* gcur, uint8_t* rec) {
     const RecFmt f = bt.hdr->fmt;
     const uint64_t cap = (uint64_t)bt.hdr->n_records;
-    const uint32_t vmask = (1u << f.sb) - 1;
     walk_batch(bt, [&](int m, const BatchMesh& M, int64_t le, int t, const int32_t* nd) {
         const int npe = npe_of(t), K = k_of(t);
         uint32_t* cur = gcur + bt.bucket_off[m];
@@ -151,23 +150,16 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_part_b(BatchTables bt, uint32
         for (int i = 0; i < 8; ++i) {
             if (pos[i] >= cap) continue;
             const int32_t v = nd[i];
-            int nf = 0;
+            uint32_t nf = 0;
 #pragma unroll
             for (int q = 0; q < 8; ++q) nf |= (q < i) && (nd[q] == v);
-            Rec r{(uint64_t)((uint32_t)v & vmask), 0};
-            if (f.want & NN_WANT_ELEMS) {
-                rec_put(r, (uint64_t)nf, f.off_nf);
-                rec_put(r, (uint64_t)le, f.off_e);
-            }
-            if (f.want & NN_WANT_NODES) {
+            uint32_t n[3];
 #pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    if (s >= K) break;
-                    const int32_t y = nbr_node(t, nd, i, s);
-                    rec_put(r, y == v ? 0ull : (uint64_t)(uint32_t)(y + 1), f.off_n + s * f.nb);
-                }
+            for (int s = 0; s < 3; ++s) {
+                const int32_t y = s < K ? nbr_node(t, nd, i, s) : v;
+                n[s] = y == v ? f.nmask : (uint32_t)y;
             }
-            reinterpret_cast<ulonglong2*>(rec)[pos[i]] = make_ulonglong2(r.lo, r.hi);
+            put_rec<16>(rec, pos[i], pack_rec<16>(f, make_side(f, (uint32_t)v, nf), (uint32_t)le, n, K));
         }
     });
 }

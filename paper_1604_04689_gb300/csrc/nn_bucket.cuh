@@ -50,22 +50,6 @@ constexpr uint32_t FULL = 0xffffffffu;
 constexpr uint32_t PREFETCH = 32768;  // bytes per prefetch instruction
 constexpr uint32_t CHAIN_END = 0xffffffffu;
 
-// ------------------------------------------------------------- records
-// Record i of the current bucket (rp points at its record 0).
-template <int RB>
-__device__ __forceinline__ Rec get_rec(const uint8_t* rp, uint32_t i) {
-    Rec x;
-    if constexpr (RB == 8) {
-        x.lo = __ldg(reinterpret_cast<const unsigned long long*>(rp) + i);
-        x.hi = 0;
-    } else {
-        const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(rp) + i);
-        x.lo = w.x;
-        x.hi = w.y;
-    }
-    return x;
-}
-
 __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
@@ -149,9 +133,9 @@ __device__ inline void warp_bitonic_sort(uint32_t* a, uint32_t n) {
 
 // The element ids of a node's c records (a repeated node's record adds
 // none), collected by its whole warp into row[0..ec) and sorted there.
-template <int RB>
-__device__ __noinline__ void warp_elem_row(const uint8_t* rp, const uint32_t* grp, uint32_t c, uint32_t* row,
-                                           uint32_t ec, int off_nf, int off_e, int eb) {
+template <int RB, int K>
+__device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, const uint32_t* grp, uint32_t c,
+                                           uint32_t* row, uint32_t ec) {
     const uint32_t lane = threadIdx.x & 31;
     uint32_t wpos = 0;
     for (uint32_t s0 = 0; s0 < c; s0 += 32) {
@@ -159,9 +143,9 @@ __device__ __noinline__ void warp_elem_row(const uint8_t* rp, const uint32_t* gr
         bool keep = false;
         uint32_t e = 0;
         if (s < c) {
-            const Rec x = get_rec<RB>(rp, grp[s]);
-            keep = !rec_get(x, off_nf, 1);
-            e = rec_get(x, off_e, eb);
+            const Rec x = load_rec<RB>(rp, grp[s]);
+            keep = !((rec_side<RB, K>(f, x) >> f.off_nf) & 1u);
+            e = rec_elem<RB>(f, x);
         }
         const unsigned km = __ballot_sync(FULL, keep);
         if (keep) row[wpos + __popc(km & lanemask_lt())] = e;
@@ -174,26 +158,26 @@ __device__ __noinline__ void warp_elem_row(const uint8_t* rp, const uint32_t* gr
 // The distinct neighbours of a node's c records, collected by its whole warp
 // into a[0 .. K c): sorted, the first of every run kept.  Returns their count.
 template <int RB, int K>
-__device__ __noinline__ uint32_t warp_node_row(const uint8_t* rp, const uint32_t* grp, uint32_t c, uint32_t* a,
-                                               int off_n, int nb) {
+__device__ __noinline__ uint32_t warp_node_row(const RecFmt& f, const uint8_t* rp, const uint32_t* grp, uint32_t c,
+                                               uint32_t* a) {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t nc = (uint64_t)K * c;
     for (uint32_t s = lane; s < c; s += 32) {
-        const Rec x = get_rec<RB>(rp, grp[s]);
+        const Rec x = load_rec<RB>(rp, grp[s]);
 #pragma unroll
-        for (int j = 0; j < K; ++j) a[(uint64_t)s * K + j] = rec_get(x, off_n + j * nb, nb) - 1;  // 0 (none) -> EMPTY
+        for (int j = 0; j < K; ++j) a[(uint64_t)s * K + j] = rec_nbr<RB>(f, x, j);
     }
     __syncwarp();
     warp_bitonic_sort(a, (uint32_t)nc);
     // keep the first of every run (in place: writes never pass the chunk being read)
-    uint32_t nu = 0, carry = EMPTY;
+    uint32_t nu = 0, carry = f.nmask;
     for (uint32_t i0 = 0; i0 < nc; i0 += 32) {
         const uint32_t idx = i0 + lane;
-        const uint32_t val = idx < nc ? a[idx] : EMPTY;
+        const uint32_t val = idx < nc ? a[idx] : f.nmask;
         uint32_t prev = __shfl_up_sync(FULL, val, 1);
         if (lane == 0) prev = carry;
         carry = __shfl_sync(FULL, val, 31);
-        const bool keep = val != EMPTY && val != prev;
+        const bool keep = val != f.nmask && val != prev;
         const unsigned km = __ballot_sync(FULL, keep);
         __syncwarp();
         if (keep) a[nu + __popc(km & lanemask_lt())] = val;
@@ -272,6 +256,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
     __shared__ uint32_t sh_list[2];   // listed records (of this bucket, of the next)
     __shared__ uint32_t sh_big[2];    // the bucket needs the whole CTA (this one, the next)
     __shared__ uint64_t sh_scan[34];
+    __shared__ RecFmt sh_fmt;         // for the out-of-line helpers
     __shared__ uint64_t sh_spill[2];  // this CTA's part of the spill area: first word, words
     const bool batched = p.batch.hdr != nullptr;
     const RecFmt f = batched ? p.batch.hdr->fmt : p.fmt;
@@ -335,6 +320,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
     clear(0);
     if (tid == 0) {
         sh_spill[0] = sh_spill[1] = 0;
+        sh_fmt = f;
         take(0, atomicAdd(p.ticket, 1u));
     }
     __syncthreads();
@@ -373,27 +359,26 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
             Rec x[U];
 #pragma unroll
             for (int q = 0; q < U; ++q)
-                if (rb + q * T + tid < R) x[q] = get_rec<RB>(rp, rb + q * T + tid);
+                if (rb + q * T + tid < R) x[q] = load_rec<RB>(rp, rb + q * T + tid);
 #pragma unroll
             for (int q = 0; q < U; ++q) {
                 if (rb + q * T + tid >= R) break;
-                const uint32_t v = (uint32_t)x[q].lo & vmask;
+                const uint32_t side = rec_side<RB, K>(f, x[q]), v = side & vmask;
                 const uint32_t s = atomicAdd(&c32[v], 1u);
-                const bool nf = want_e && rec_get(x[q], f.off_nf, 1);
+                const bool nf = want_e && ((side >> f.off_nf) & 1u);
                 if (nf) atomicAdd(&nfc[v], 1u);
                 if (s < (uint32_t)C) {
                     uint32_t* const col = table + ((v >> 5) * (uint32_t)GW + (v & 31));
-                    if (want_e) col[s * 32] = nf ? EMPTY : rec_get(x[q], f.off_e, f.eb);
+                    if (want_e) col[s * 32] = nf ? EMPTY : rec_elem<RB>(f, x[q]);
                     if (want_n) {
 #pragma unroll
                         for (int j = 0; j < K; ++j)
-                            col[(EC + s * K + j) * 32] = rec_get(x[q], f.off_n + j * f.nb, f.nb) - 1;  // none -> EMPTY
+                            col[(EC + s * K + j) * 32] = rec_nbr<RB>(f, x[q], j);
                     }
                 } else {
                     const uint32_t i = atomicAdd(&sh_list[cur], 1u);
                     if (i < (uint32_t)p.list_cap && s < (uint32_t)VE) {
-                        if constexpr (RB == 8) reinterpret_cast<uint64_t*>(list)[i] = x[q].lo;
-                        else reinterpret_cast<ulonglong2*>(list)[i] = make_ulonglong2(x[q].lo, x[q].hi);
+                        put_rec<RB>(list, i, x[q]);
                         link[i] = (uint16_t)atomicExch(&first[v], i);
                     } else {
                         sh_big[cur] = 1;
@@ -410,18 +395,6 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
         const int nb = (int)(N - v0 < (int64_t)NB ? N - v0 : (int64_t)NB);
         const bool e_ok = want_e && M.ge + M.ne <= (uint64_t)sh_out.cap_e;
         if (want_e && !e_ok && tid == 0) set_status(status, NN_ERR_CAPACITY);
-        auto list_rec = [&](uint32_t i) {
-            Rec x;
-            if constexpr (RB == 8) {
-                x.lo = reinterpret_cast<const uint64_t*>(list)[i];
-                x.hi = 0;
-            } else {
-                const ulonglong2 w = reinterpret_cast<const ulonglong2*>(list)[i];
-                x.lo = w.x;
-                x.hi = w.y;
-            }
-            return x;
-        };
         auto next_of = [&](uint32_t i) {
             const uint32_t n = link[i];
             return n == 0xffffu ? CHAIN_END : n;
@@ -445,11 +418,12 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
             uint32_t* const ncol = ecol + EC * 32;
             // 2a. neighbour row
             if (want_n) {
+                const uint32_t none = f.nmask;  // above every id: sorts last
                 uint32_t w[NW];
                 const uint32_t mine = min(c, (uint32_t)C);
                 uint32_t nw = K * tmax;
 #pragma unroll
-                for (int i = 0; i < NW; ++i) w[i] = EMPTY;
+                for (int i = 0; i < NW; ++i) w[i] = none;
 #pragma unroll
                 for (int s0 = 0; s0 < IMAX; s0 += 4) {
                     if ((uint32_t)s0 >= tmax) break;
@@ -465,13 +439,13 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
                     sort_prefix(w, nw);
                     // distinct values to the front of the lane's column
                     uint32_t* d = ncol;
-                    if (w[0] != EMPTY) *d = w[0], d += 32;
+                    if (w[0] != none) *d = w[0], d += 32;
 #pragma unroll
                     for (int i0 = 1; i0 < NW; i0 += 6) {
                         if ((uint32_t)i0 >= nw) break;
 #pragma unroll
                         for (int i = i0; i < i0 + 6 && i < NW; ++i)
-                            if (w[i] != EMPTY && w[i] != w[i - 1]) *d = w[i], d += 32;
+                            if (w[i] != none && w[i] != w[i - 1]) *d = w[i], d += 32;
                     }
                     u = (uint32_t)(d - ncol) / 32;
                     if (!__any_sync(FULL, at != CHAIN_END)) break;
@@ -482,15 +456,15 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
                         at = CHAIN_END;
                     }
                     while (at != CHAIN_END && u + K <= (uint32_t)NC) {
-                        const Rec x = list_rec(at);
+                        const Rec x = take_rec<RB>(list, at);
                         at = next_of(at);
 #pragma unroll
-                        for (int j = 0; j < K; ++j) ncol[(u + j) * 32] = rec_get(x, f.off_n + j * f.nb, f.nb) - 1;
+                        for (int j = 0; j < K; ++j) ncol[(u + j) * 32] = rec_nbr<RB>(f, x, j);
                         u += K;
                     }
                     nw = __reduce_max_sync(FULL, u);
 #pragma unroll
-                    for (int i = 0; i < NW; ++i) w[i] = (uint32_t)i < u ? ncol[i * 32] : EMPTY;
+                    for (int i = 0; i < NW; ++i) w[i] = (uint32_t)i < u ? ncol[i * 32] : none;
                 }
                 const uint32_t umax = __reduce_max_sync(FULL, u);
 #pragma unroll
@@ -544,9 +518,9 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
 #pragma unroll
                     for (int s = 0; s < VE; ++s) {
                         if (s >= C && at != CHAIN_END) {
-                            const Rec x = list_rec(at);
+                            const Rec x = take_rec<RB>(list, at);
                             at = next_of(at);
-                            if (!rec_get(x, f.off_nf, 1)) v[s] = rec_get(x, f.off_e, f.eb);
+                            if (!((rec_side<RB, K>(f, x) >> f.off_nf) & 1u)) v[s] = rec_elem<RB>(f, x);
                         }
                     }
                 }
@@ -621,7 +595,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
         const bool ok = sh_spill[1] >= need;
         uint32_t* const grp = p.spill + sh_spill[0];
         for (uint32_t r = tid; ok && r < R; r += T)
-            grp[atomicAdd(&cursor[(uint32_t)get_rec<RB>(rp, r).lo & vmask], 1u)] = r;
+            grp[atomicAdd(&cursor[rec_side<RB, K>(f, load_rec<RB>(rp, r)) & vmask], 1u)] = r;
         __syncthreads();
         uint32_t* const scratch = table + 2 * NB + warp * scratch_words;
         for (int g = warp; g < GP; g += W) {
@@ -635,7 +609,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
                 if (want_e) {
                     if (lane == 0 && NN_IN(v0 + l, N + 1, status)) sh_out.rp_e[v0 + l] = (int64_t)(M.ge + eoff[l]);
                     if (ok && e_ok && c) {
-                        warp_elem_row<RB>(rp, grp + o, c, a, ec, f.off_nf, f.off_e, f.eb);
+                        warp_elem_row<RB, K>(sh_fmt, rp, grp + o, c, a, ec);
                         for (uint32_t k = lane; k < ec; k += 32) sh_out.col_e[M.ge + eoff[l] + k] = (int32_t)a[k];
                         __syncwarp();
                     }
@@ -643,7 +617,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
                 if (want_n) {
                     uint32_t u = 0;
                     if (ok && c) {
-                        u = warp_node_row<RB, K>(rp, grp + o, c, a, f.off_n, f.nb);
+                        u = warp_node_row<RB, K>(sh_fmt, rp, grp + o, c, a);
                         const size_t d = (size_t)K * (M.r0 + pr) + run;
                         if (u == 0 || NN_IN(d + u - 1, p.ntmp_words, status))
                             for (uint32_t k = lane; k < u; k += 32) p.ntmp[d + k] = a[k];

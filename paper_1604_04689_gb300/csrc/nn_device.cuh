@@ -158,28 +158,99 @@ __device__ inline uint64_t smem_array_excl_scan(uint64_t* a, int n, uint64_t* sh
 }
 
 // --------------------------------------------------------------- records
+// (the layout is described at RecFmt; 8-byte records use x and y)
 struct Rec {
-    uint64_t lo, hi;
+    uint32_t x, y, z, w;
 };
 
-__device__ __forceinline__ void rec_put(Rec& r, uint64_t val, int off) {  // val < 2^32
-    if (off < 64) {
-        r.lo |= val << off;
-        if (off > 32) r.hi |= val >> (64 - off);
+// The side of a node at vr (relative to the build's first node).
+__device__ __forceinline__ uint32_t make_side(const RecFmt& f, uint32_t vr, uint32_t nf) {
+    const int bits = f.sb + (f.cshift > 0 ? f.cshift : 0);
+    return (vr & ((1u << bits) - 1u)) | ((f.want & NN_WANT_ELEMS) ? nf << f.off_nf : 0u);
+}
+// n: the neighbours, f.nmask for none (n[2] is not used when k = 2)
+template <int RB>
+__device__ __forceinline__ Rec pack_rec(const RecFmt& f, uint32_t side, uint32_t e, const uint32_t (&n)[3], int K) {
+    Rec r;
+    if constexpr (RB == 8) {
+        uint64_t v = side;
+        if (f.want & NN_WANT_ELEMS) v |= (uint64_t)e << f.off_e;
+        if (f.want & NN_WANT_NODES) {
+            v |= (uint64_t)n[0] << f.off_n;
+            v |= (uint64_t)n[1] << (f.off_n + f.nb);
+            if (f.k == 3) v |= (uint64_t)(K == 3 ? n[2] : f.nmask) << (f.off_n + 2 * f.nb);
+        }
+        r = Rec{(uint32_t)v, (uint32_t)(v >> 32), 0u, 0u};
     } else {
-        r.hi |= val << (off - 64);
+        const uint32_t n2 = f.k == 3 ? (K == 3 ? n[2] : f.nmask) : 0u;
+        r = Rec{e, n[0], n[1], n2};
+        if (f.side_split) {
+            r.y |= side << f.nb;
+            r.z |= (side >> f.sh2) << f.nb;
+            r.w |= (side >> f.sh3) << f.nb;
+            r.x |= (side >> f.sh0) << f.eb;
+        } else if (f.k == 2 || !(f.want & NN_WANT_NODES)) {
+            r.w = side;
+        } else {
+            r.x = side;
+        }
+    }
+    return r;
+}
+// The side; bits above it may be set in 8-byte records.  K: f.k where the
+// caller knows it at compile time (0: look it up).
+template <int RB, int K>
+__device__ __forceinline__ uint32_t rec_side(const RecFmt& f, const Rec& r) {
+    if constexpr (RB == 8) {
+        return r.x;
+    } else if constexpr (K == 2) {
+        return r.w;
+    } else {
+        if (f.side_split)
+            return (r.y >> f.nb) | ((r.z >> f.nb) << f.sh2) | ((r.w >> f.nb) << f.sh3) | ((r.x >> f.eb) << f.sh0);
+        return (K == 0 && f.k == 2) || !(f.want & NN_WANT_NODES) ? r.w : r.x;
     }
 }
-// Field of `width` <= 32 bits at bit `off` of the 128-bit record (no field
-// crosses bit 128).  Branch-free: the field starts in 32-bit word off / 32
-// and a funnel shift takes it across into the next word.
-__device__ __forceinline__ uint32_t rec_get(const Rec& r, int off, int width) {
-    const uint32_t w0 = (uint32_t)r.lo, w1 = (uint32_t)(r.lo >> 32), w2 = (uint32_t)r.hi, w3 = (uint32_t)(r.hi >> 32);
-    const int q = off >> 5;
-    const uint32_t a = q == 0 ? w0 : (q == 1 ? w1 : (q == 2 ? w2 : w3));
-    const uint32_t b = q == 0 ? w1 : (q == 1 ? w2 : (q == 2 ? w3 : 0u));
-    const uint32_t v = __funnelshift_r(a, b, (uint32_t)off & 31u);
-    return width >= 32 ? v : v & ((1u << width) - 1u);
+// 32 bits of an 8-byte record from bit off < 64
+__device__ __forceinline__ uint32_t rec_bits(const Rec& r, int off) {
+    return off < 32 ? __funnelshift_r(r.x, r.y, (uint32_t)off) : r.y >> (off - 32);
+}
+template <int RB>
+__device__ __forceinline__ uint32_t rec_elem(const RecFmt& f, const Rec& r) {
+    if constexpr (RB == 8) return rec_bits(r, f.off_e) & f.emask;
+    else return r.x & f.emask;
+}
+// neighbour j (f.nmask: none)
+template <int RB>
+__device__ __forceinline__ uint32_t rec_nbr(const RecFmt& f, const Rec& r, int j) {
+    if constexpr (RB == 8) return rec_bits(r, f.off_n + j * f.nb) & f.nmask;
+    else return (j == 0 ? r.y : (j == 1 ? r.z : r.w)) & f.nmask;
+}
+template <int RB>
+__device__ __forceinline__ void put_rec(uint8_t* base, uint64_t pos, const Rec& r) {
+    if constexpr (RB == 8) reinterpret_cast<uint2*>(base)[pos] = make_uint2(r.x, r.y);
+    else reinterpret_cast<uint4*>(base)[pos] = make_uint4(r.x, r.y, r.z, r.w);
+}
+template <int RB>
+__device__ __forceinline__ Rec take_rec(const uint8_t* base, uint64_t pos) {
+    if constexpr (RB == 8) {
+        const uint2 v = reinterpret_cast<const uint2*>(base)[pos];
+        return Rec{v.x, v.y, 0u, 0u};
+    } else {
+        const uint4 v = reinterpret_cast<const uint4*>(base)[pos];
+        return Rec{v.x, v.y, v.z, v.w};
+    }
+}
+// Read-only global memory (written by an earlier kernel).
+template <int RB>
+__device__ __forceinline__ Rec load_rec(const uint8_t* base, uint64_t pos) {
+    if constexpr (RB == 8) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(base) + pos);
+        return Rec{v.x, v.y, 0u, 0u};
+    } else {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(base) + pos);
+        return Rec{v.x, v.y, v.z, v.w};
+    }
 }
 
 // ------------------------------------------------ element local edge tables

@@ -281,12 +281,32 @@ struct PartShape {
     static constexpr int UPT = (TYPE == NN_TRI) ? 1 : (NPE == 8 ? 2 : 3);  // units per thread per round
 };
 
+// The record of local node i of element e (of run-time type t), whose nodes
+// are e_nd; vr: the node's id relative to the build's first node.
+template <int TYPE, int RB>
+__device__ __forceinline__ Rec make_rec(const RecFmt& f, const int32_t* e_nd, int i, int t, uint32_t e, uint32_t vr) {
+    constexpr int NPE = PartShape<TYPE>::NPE;
+    const int32_t v = e_nd[i];
+    uint32_t nf = 0;
+#pragma unroll
+    for (int q = 0; q < NPE; ++q) nf |= (q < i) && (e_nd[q] == v);
+    const int K = TYPE == NN_MIXED ? k_of(t) : ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::K;
+    uint32_t n[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        int32_t y = v;
+        if (s < K)
+            y = TYPE == NN_MIXED ? nbr_node(t, e_nd, i, s) : e_nd[ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::nbr(i, s)];
+        n[s] = y == v ? f.nmask : (uint32_t)y;
+    }
+    return pack_rec<RB>(f, make_side(f, vr, nf), e, n, K);
+}
+
 template <int TYPE, int RB, bool RANGED>
 __global__ void __launch_bounds__(PART_THREADS, 2) k_part(EmitParams p) {
     using S = PartShape<TYPE>;
     constexpr int UNIT = S::UNIT, NPE = S::NPE, UPT = S::UPT, NI = NPE * UNIT;
     const RecFmt f = p.fmt;
-    const uint32_t vmask = (1u << f.sb) - 1;
     const int64_t n_units = (p.n_elems + UNIT - 1) / UNIT;
     const int64_t u0 = n_units * blockIdx.x / gridDim.x, u1 = n_units * (blockIdx.x + 1) / gridDim.x;
     for (int64_t ub = u0 + (int64_t)threadIdx.x * UPT; ub < u1; ub += (int64_t)blockDim.x * UPT) {
@@ -321,33 +341,9 @@ __global__ void __launch_bounds__(PART_THREADS, 2) k_part(EmitParams p) {
                 const int w = j / NPE, i = j % NPE;
                 if (pos[k][j] >= p.rec_cap) continue;  // not an incidence, or overlapping invalid mixed elements
                 const int32_t* e_nd = nd[k] + w * NPE;
-                const int32_t v = e_nd[i];
-                int nf = 0;
-#pragma unroll
-                for (int q = 0; q < NPE; ++q) nf |= (q < i) && (e_nd[q] == v);
-                const int K = TYPE == NN_MIXED ? k_of(tk) : ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::K;
                 uint32_t vr;
-                node_in<RANGED>(p, v, vr);
-                Rec r{(uint64_t)(vr & vmask), 0};
-                if (f.want & NN_WANT_ELEMS) {
-                    rec_put(r, (uint64_t)nf, f.off_nf);
-                    rec_put(r, (uint64_t)((ub + k) * UNIT + w), f.off_e);
-                }
-                if (f.want & NN_WANT_NODES) {
-#pragma unroll
-                    for (int s = 0; s < 3; ++s) {
-                        if (s >= K) break;
-                        const int32_t y = TYPE == NN_MIXED
-                                              ? nbr_node(tk, e_nd, i, s)
-                                              : e_nd[ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::nbr(i, s)];
-                        rec_put(r, y == v ? 0ull : (uint64_t)(uint32_t)(y + 1), f.off_n + s * f.nb);
-                    }
-                }
-                if constexpr (RB == 8) {
-                    reinterpret_cast<uint64_t*>(p.rec)[pos[k][j]] = r.lo;
-                } else {
-                    reinterpret_cast<ulonglong2*>(p.rec)[pos[k][j]] = make_ulonglong2(r.lo, r.hi);
-                }
+                node_in<RANGED>(p, e_nd[i], vr);
+                put_rec<RB>(p.rec, pos[k][j], make_rec<TYPE, RB>(f, e_nd, i, tk, (uint32_t)((ub + k) * UNIT + w), vr));
             }
         }
     }
@@ -399,8 +395,8 @@ struct SortShape {
 };
 
 template <int TYPE>
-__host__ __device__ constexpr size_t coarse_smem() {
-    return (size_t)SortShape<TYPE>::TILE * 17 + 3 * 256 * 4;
+__host__ __device__ constexpr size_t coarse_smem(int rb) {
+    return (size_t)SortShape<TYPE>::TILE * (rb + 1) + 3 * 256 * 4;
 }
 // Records per thread of a fine-pass tile: 4, or 8 when a coarse region has
 // at least 512 buckets (then a 1024-record tile has about two records per
@@ -415,48 +411,10 @@ constexpr int FINE_DIGITS = 4096;  // buckets per coarse region: at most 256 x 4
 // per-digit tables and the first work item of every coarse region
 __host__ __device__ constexpr size_t fine_stage_bytes(int tile, int rb) { return (size_t)tile * rb + 16; }
 __host__ __device__ constexpr size_t fine_smem(int nd, int rb) {
-    return 2 * fine_stage_bytes(SORT_THREADS * fine_rpt(nd), rb) + (size_t)SORT_THREADS * fine_rpt(nd) * 18 +
+    return 2 * fine_stage_bytes(SORT_THREADS * fine_rpt(nd), rb) + (size_t)SORT_THREADS * fine_rpt(nd) * (rb + 2) +
            3 * (size_t)nd * 4 + 257 * 4;
 }
 constexpr size_t FINE_SMEM = fine_smem(FINE_DIGITS, 16);
-
-// vr: the node's id relative to the build's first node
-template <int TYPE>
-__device__ __forceinline__ Rec make_rec(const RecFmt& f, const int32_t* e_nd, int i, int t, int64_t e, uint32_t vr) {
-    constexpr int NPE = SortShape<TYPE>::NPE;
-    const int32_t v = e_nd[i];
-    int nf = 0;
-#pragma unroll
-    for (int q = 0; q < NPE; ++q) nf |= (q < i) && (e_nd[q] == v);
-    const int K = TYPE == NN_MIXED ? k_of(t) : ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::K;
-    Rec r{(uint64_t)(vr & ((1u << f.sb) - 1)), 0};
-    if (f.want & NN_WANT_ELEMS) {
-        rec_put(r, (uint64_t)nf, f.off_nf);
-        rec_put(r, (uint64_t)e, f.off_e);
-    }
-    if (f.want & NN_WANT_NODES) {
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            if (s >= K) break;
-            const int32_t y = TYPE == NN_MIXED ? nbr_node(t, e_nd, i, s)
-                                               : e_nd[ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::nbr(i, s)];
-            rec_put(r, y == v ? 0ull : (uint64_t)(uint32_t)(y + 1), f.off_n + s * f.nb);
-        }
-    }
-    if (f.cshift > 0) rec_put(r, (uint64_t)((vr >> f.sb) & ((1u << f.cshift) - 1)), f.off_fb);
-    return r;
-}
-
-template <int RB>
-__device__ __forceinline__ void store_rec(uint8_t* base, uint64_t pos, const ulonglong2& r) {
-    if constexpr (RB == 8) reinterpret_cast<uint64_t*>(base)[pos] = r.x;
-    else reinterpret_cast<ulonglong2*>(base)[pos] = r;
-}
-template <int RB>
-__device__ __forceinline__ ulonglong2 load_rec2(const uint8_t* base, uint64_t pos) {
-    if constexpr (RB == 8) return make_ulonglong2(__ldg(reinterpret_cast<const unsigned long long*>(base) + pos), 0);
-    else return __ldg(reinterpret_cast<const ulonglong2*>(base) + pos);
-}
 
 // First (or only) pass: records from the connectivity, radix digit = coarse
 // region (two levels) or bucket (one level, at most 256 buckets).
@@ -465,8 +423,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
     using S = SortShape<TYPE>;
     constexpr int UNIT = S::UNIT, NPE = S::NPE, UPT = S::UPT, NI = S::NI, TILE = S::TILE;
     extern __shared__ __align__(16) uint8_t sm[];
-    ulonglong2* out = reinterpret_cast<ulonglong2*>(sm);
-    uint8_t* odig = reinterpret_cast<uint8_t*>(out + TILE);
+    uint8_t* odig = sm + (size_t)TILE * RB;
     uint32_t* hist = reinterpret_cast<uint32_t*>(odig + TILE);
     uint32_t* dof = hist + 256;
     uint32_t* gbase = dof + 256;
@@ -519,9 +476,8 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
                 const int w = j / NPE, i = j % NPE;
                 uint32_t vr;
                 node_in<RANGED>(p, nd[k][j], vr);
-                const Rec r = make_rec<TYPE>(f, nd[k] + w * NPE, i, t[k], u * UNIT + w, vr);
                 const uint32_t q = dof[dg[k][j]] + rk[k][j];
-                out[q] = make_ulonglong2(r.lo, r.hi);
+                put_rec<RB>(sm, q, make_rec<TYPE, RB>(f, nd[k] + w * NPE, i, t[k], (uint32_t)(u * UNIT + w), vr));
                 odig[q] = dg[k][j];
             }
         }
@@ -529,7 +485,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
         for (uint32_t q = threadIdx.x; q < n_tile; q += SORT_THREADS) {
             const uint32_t d = odig[q];
             const uint64_t pos = (uint64_t)gbase[d] + (q - dof[d]);
-            if (pos < p.rec_cap) store_rec<RB>(dst, pos, out[q]);
+            if (pos < p.rec_cap) put_rec<RB>(dst, pos, take_rec<RB>(sm, q));
         }
         __syncthreads();
     }
@@ -547,8 +503,8 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr uint32_t SB = (uint32_t)fine_stage_bytes(FINE_TILE, RB);
     uint8_t* const stage = sm;  // [2][SB]
-    ulonglong2* out = reinterpret_cast<ulonglong2*>(sm + 2 * SB);
-    uint16_t* odig = reinterpret_cast<uint16_t*>(out + FINE_TILE);
+    uint8_t* out = sm + 2 * SB;
+    uint16_t* odig = reinterpret_cast<uint16_t*>(out + (size_t)FINE_TILE * RB);
     const RecFmt f = p.fmt;
     const int cs = f.cshift;
     const int nd_ = 1 << cs;  // digits (buckets) per coarse region, <= FINE_DIGITS
@@ -637,12 +593,8 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         // a thread keeps its records' digits and ranks, and the records
         // themselves in registers when it holds four (else they are read
         // from the stage again when placed)
-        auto rec_at = [&](uint32_t r) {
-            if constexpr (RB == 8) return make_ulonglong2(reinterpret_cast<const unsigned long long*>(src)[r], 0);
-            else return reinterpret_cast<const ulonglong2*>(src)[r];
-        };
         constexpr int XR = FINE_RPT <= 4 ? FINE_RPT : 1;
-        ulonglong2 x[XR];
+        Rec x[XR];
         uint16_t rk[FINE_RPT];
         uint16_t dg[FINE_RPT];
 #pragma unroll
@@ -651,10 +603,9 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
             rk[k] = 0xFFFF;
             dg[k] = 0;
             if (r < n) {
-                const ulonglong2 xr = rec_at(r);
+                const Rec xr = take_rec<RB>(src, r);
                 if constexpr (FINE_RPT <= 4) x[k] = xr;
-                const Rec rr{xr.x, xr.y};
-                dg[k] = (uint16_t)rec_get(rr, f.off_fb, cs);
+                dg[k] = (uint16_t)((rec_side<RB, 0>(f, xr) >> f.sb) & (uint32_t)(nd_ - 1));
             }
         }
 #pragma unroll
@@ -668,15 +619,15 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         for (int k = 0; k < FINE_RPT; ++k) {
             if (rk[k] == 0xFFFF) continue;
             const uint32_t q = dof[dg[k]] + rk[k];
-            if constexpr (FINE_RPT <= 4) out[q] = x[k];
-            else out[q] = rec_at(threadIdx.x + k * SORT_THREADS);
+            if constexpr (FINE_RPT <= 4) put_rec<RB>(out, q, x[k]);
+            else put_rec<RB>(out, q, take_rec<RB>(src, threadIdx.x + k * SORT_THREADS));
             odig[q] = dg[k];
         }
         __syncthreads();
         for (uint32_t q = threadIdx.x; q < n_tile; q += SORT_THREADS) {
             const uint32_t dd = odig[q];
             const uint64_t pos = (uint64_t)gbase[dd] + (q - dof[dd]);
-            if (pos < p.rec_cap) store_rec<RB>(p.rec, pos, out[q]);
+            if (pos < p.rec_cap) put_rec<RB>(p.rec, pos, take_rec<RB>(out, q));
         }
         __syncthreads();
     }
@@ -750,7 +701,7 @@ cudaError_t part_t(const EmitParams& p, cudaStream_t s) {
 
 template <int TYPE>
 cudaError_t set_sorted_smem() {
-    const int b = (int)coarse_smem<TYPE>();
+    const int b = (int)coarse_smem<TYPE>(16);
     cudaError_t e = cudaFuncSetAttribute(k_part_coarse<TYPE, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_part_coarse<TYPE, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
@@ -793,7 +744,7 @@ cudaError_t launch_part(const EmitParams& p, cudaStream_t s) {
 
 template <int TYPE, bool RANGED>
 void coarse_r(const EmitParams& p, cudaStream_t s) {
-    const size_t smem = coarse_smem<TYPE>();
+    const size_t smem = coarse_smem<TYPE>(p.fmt.rb);
     if (p.fmt.rb == 8) k_part_coarse<TYPE, 8, RANGED><<<p.n_cta_part, SORT_THREADS, smem, s>>>(p);
     else k_part_coarse<TYPE, 16, RANGED><<<p.n_cta_part, SORT_THREADS, smem, s>>>(p);
 }
