@@ -356,23 +356,6 @@ __global__ void __launch_bounds__(PART_THREADS, 2) k_part(EmitParams p) {
 // contiguously, so global stores are coalesced runs instead of one scattered
 // 16-byte store per record.
 
-// Exclusive scan of hist[0..n) (any n) into dof, a contiguous chunk per thread;
-// returns the total.  Ends with a barrier: any thread may read any dof entry.
-__device__ __forceinline__ uint32_t tile_scan_n(const uint32_t* hist, uint32_t* dof, int n, uint64_t* sh) {
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int lo = min(n, (int)threadIdx.x * per), hi = min(n, lo + per);
-    uint64_t x = 0;
-    for (int i = lo; i < hi; ++i) x += hist[i];
-    uint64_t total;
-    uint64_t run = block_excl_scan(x, &total, sh);
-    for (int i = lo; i < hi; ++i) {
-        dof[i] = (uint32_t)run;
-        run += hist[i];
-    }
-    __syncthreads();
-    return (uint32_t)total;
-}
-
 // Exclusive scan of hist[0..n) (n <= blockDim.x) into dof; returns the total.
 // Ends with a barrier: every thread may read any dof entry afterwards.
 __device__ __forceinline__ uint32_t tile_scan(const uint32_t* hist, uint32_t* dof, int n, uint64_t* sh) {
@@ -407,12 +390,12 @@ __host__ __device__ constexpr int fine_rpt(int nd) { return nd >= FINE_RPT_WIDE_
 constexpr int FINE_DIGITS = 4096;  // buckets per coarse region: at most 256 x 4096 buckets in all
 // shared memory of the fine pass for nd digits per coarse region and rb-byte
 // records: two tile stages (bulk-copy targets, 16 bytes of slack for an odd
-// 8-byte first record), the tile in digit order with its digits, three
-// per-digit tables and the first work item of every coarse region
+// 8-byte first record), the tile's order, three per-digit tables and the
+// first work item and record of every coarse region
 __host__ __device__ constexpr size_t fine_stage_bytes(int tile, int rb) { return (size_t)tile * rb + 16; }
 __host__ __device__ constexpr size_t fine_smem(int nd, int rb) {
-    return 2 * fine_stage_bytes(SORT_THREADS * fine_rpt(nd), rb) + (size_t)SORT_THREADS * fine_rpt(nd) * (rb + 2) +
-           3 * (size_t)nd * 4 + 257 * 4;
+    return 2 * fine_stage_bytes(SORT_THREADS * fine_rpt(nd), rb) + (size_t)SORT_THREADS * fine_rpt(nd) * 2 +
+           3 * (size_t)nd * 4 + 2 * 257 * 4;
 }
 constexpr size_t FINE_SMEM = fine_smem(FINE_DIGITS, 16);
 
@@ -497,50 +480,65 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
 // memory by a bulk asynchronous copy issued while the CTA still sorts and
 // writes the tile before it (two stages, one mbarrier each, bounded waits),
 // so the tile loads overlap the in-tile sort instead of stalling it.
-template <int RB, int FINE_RPT>
+//
+// What bounds it: the barriers between a tile's short phases, then its
+// partly filled lines on the way out.  The records stay where the copy put
+// them (a 16-bit index per place orders them), a thread scans the digits that
+// it clears and reserves, the cursors' atomics are in flight while the tile is
+// put in order, and the regions' bounds are kept in shared memory for the
+// thread that starts the copies.  DPT: digits a thread may own (their
+// reservations are held in registers: one size for all cost a third of the
+// resident CTAs).  GB300, before and now: tet 161^3 0.71 -> 0.50 ms (6.3 TB/s
+// read and written), triangles 2048^2 0.172 -> 0.127 ms (6.0 TB/s), hex 257^3
+// (512 digits per region) 1.33 -> 0.94 ms (4.6 TB/s).
+template <int RB, int FINE_RPT, int DPT>
 __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const uint32_t* bstart) {
     constexpr int FINE_TILE = SORT_THREADS * FINE_RPT;
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr uint32_t SB = (uint32_t)fine_stage_bytes(FINE_TILE, RB);
     uint8_t* const stage = sm;  // [2][SB]
-    uint8_t* out = sm + 2 * SB;
-    uint16_t* odig = reinterpret_cast<uint16_t*>(out + (size_t)FINE_TILE * RB);
     const RecFmt f = p.fmt;
     const int cs = f.cshift;
     const int nd_ = 1 << cs;  // digits (buckets) per coarse region, <= FINE_DIGITS
-    uint32_t* hist = reinterpret_cast<uint32_t*>(odig + FINE_TILE);
-    uint32_t* dof = hist + nd_;
-    uint32_t* gbase = dof + nd_;
-    uint32_t* tpre = gbase + nd_;  // [257] first tile of each coarse region
+    uint16_t* const perm = reinterpret_cast<uint16_t*>(sm + 2 * SB);  // [FINE_TILE] record at each place
+    uint32_t* const hist = reinterpret_cast<uint32_t*>(perm + FINE_TILE);  // [nd_]
+    uint32_t* const dof = hist + nd_;     // [nd_] first place of each digit
+    uint32_t* const delta = dof + nd_;    // [nd_] global position less place
+    uint32_t* const tpre = delta + nd_;   // [257] first tile of each coarse region
+    uint32_t* const rbeg = tpre + 257;    // [257] first record of each coarse region
     __shared__ uint64_t sh_scan[34];
+    __shared__ uint32_t sh_warp[SORT_THREADS / 32];
     __shared__ uint64_t mbar[2];
     __shared__ uint32_t sh_tile[2][4];  // per stage: region, first record, end, offset of record 0 in the stage
     __shared__ int32_t sh_lost;
     const int64_t B = p.n_buckets;
     const int R1 = (int)((B + (1ll << cs) - 1) >> cs);
-    const int d0 = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t my_tiles = 0;
-    if (d0 < R1) {
-        const uint32_t a = bstart[(int64_t)d0 << cs];
-        const int64_t e_ = ((int64_t)d0 + 1) << cs;
+    if (tid < R1) {
+        const uint32_t a = bstart[(int64_t)tid << cs];
+        const int64_t e_ = ((int64_t)tid + 1) << cs;
         const uint32_t b = bstart[e_ < B ? e_ : B];
         my_tiles = (b - a + FINE_TILE - 1) / FINE_TILE;
+        rbeg[tid] = a;
+        if (tid == R1 - 1) rbeg[R1] = b;
     }
     {
         uint64_t total;
         const uint64_t ex = block_excl_scan(my_tiles, &total, sh_scan);
-        if (d0 < R1) tpre[d0] = (uint32_t)ex;
-        if (d0 == 0) tpre[R1] = (uint32_t)total;
+        if (tid < R1) tpre[tid] = (uint32_t)ex;
+        if (tid == 0) tpre[R1] = (uint32_t)total;
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         mbar_init(&mbar[0]);
         mbar_init(&mbar[1]);
         sh_lost = 0;
     }
+    for (int i = tid; i < nd_; i += SORT_THREADS) hist[i] = 0;
     __syncthreads();
     const uint32_t W = tpre[R1];
     // One thread: locate work item wi and start the copy of its records
-    // into stage st (stage st is free: its previous tile passed a barrier).
+    // into stage st (stage st is free: every thread is past its previous tile).
     auto issue = [&](int st, uint32_t wi) {
         int lo = 0, hi = R1;  // largest d with tpre[d] <= wi
         while (hi - lo > 1) {
@@ -548,14 +546,10 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
             if (tpre[mid] <= wi) lo = mid;
             else hi = mid;
         }
-        const int d = lo;
-        const int64_t fb0 = (int64_t)d << cs;
-        const int64_t fe = fb0 + (1ll << cs);
-        const uint32_t ra = bstart[fb0], rb_ = bstart[fe < B ? fe : B];
-        const uint32_t r0 = ra + (wi - tpre[d]) * FINE_TILE;
-        const uint32_t r1 = min(r0 + (uint32_t)FINE_TILE, rb_);
+        const uint32_t r0 = rbeg[lo] + (wi - tpre[lo]) * FINE_TILE;
+        const uint32_t r1 = min(r0 + (uint32_t)FINE_TILE, rbeg[lo + 1]);
         const uint32_t roff = RB == 8 ? (r0 & 1u) * 8u : 0u;
-        sh_tile[st][0] = (uint32_t)d;
+        sh_tile[st][0] = (uint32_t)lo;
         sh_tile[st][1] = r0;
         sh_tile[st][2] = r1;
         sh_tile[st][3] = roff;
@@ -567,76 +561,106 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
             bulk_load(stage + st * SB, p.rec_tmp + (uint64_t)r0 * RB - roff, bytes, &mbar[st]);
         }
     };
-    if (threadIdx.x == 0 && blockIdx.x < W) issue(0, blockIdx.x);
+    if (tid == 0 && blockIdx.x < W) issue(0, blockIdx.x);
+    const int per = nd_ > SORT_THREADS ? nd_ / SORT_THREADS : 1;  // digits of a thread (both are powers of two)
     uint32_t par[2] = {0u, 0u};  // parity of each stage's next copy
     int it = 0;
     for (uint32_t wi = blockIdx.x; wi < W; wi += gridDim.x, ++it) {
         const int st = it & 1;
-        // the next tile of this CTA, into the other stage
-        if (threadIdx.x == 0 && wi + gridDim.x < W) issue(st ^ 1, wi + gridDim.x);
-        for (int i = threadIdx.x; i < nd_; i += SORT_THREADS) hist[i] = 0;
-        // thread 0 issued this stage's copy and waits for it; the others wait
+        // thread 0, which issued this stage's copy, waits for it, the others
         // at the barrier, after which the stage's records and bounds are seen
-        if (threadIdx.x == 0 && sh_tile[st][2] > sh_tile[st][1]) {
+        // and the other stage is free: its next tile is on its way
+        if (tid == 0 && sh_tile[st][2] > sh_tile[st][1]) {
             if (!mbar_wait(&mbar[st], par[st])) sh_lost = 1;
             par[st] ^= 1u;
         }
         __syncthreads();
+        if (tid == 0 && wi + gridDim.x < W && !sh_lost) issue(st ^ 1, wi + gridDim.x);
         if (sh_lost) {  // a copy that never completed (bounded wait): report and stop
-            if (threadIdx.x == 0) set_status(p.status, NN_ERR_TIMEOUT);
+            if (tid == 0) set_status(p.status, NN_ERR_TIMEOUT);
             return;
         }
-        const int d = (int)sh_tile[st][0];
-        const int64_t fb0 = (int64_t)d << cs;
+        const int64_t fb0 = (int64_t)sh_tile[st][0] << cs;
         const uint32_t n = sh_tile[st][2] - sh_tile[st][1];
         const uint8_t* const src = stage + st * SB + sh_tile[st][3];
-        // a thread keeps its records' digits and ranks, and the records
-        // themselves in registers when it holds four (else they are read
-        // from the stage again when placed)
-        constexpr int XR = FINE_RPT <= 4 ? FINE_RPT : 1;
-        Rec x[XR];
-        uint16_t rk[FINE_RPT];
-        uint16_t dg[FINE_RPT];
+        // each record's digit and rank among its digit's records
+        uint32_t dr[FINE_RPT];
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k) {
-            const uint32_t r = threadIdx.x + k * SORT_THREADS;
-            rk[k] = 0xFFFF;
-            dg[k] = 0;
-            if (r < n) {
-                const Rec xr = take_rec<RB>(src, r);
-                if constexpr (FINE_RPT <= 4) x[k] = xr;
-                dg[k] = (uint16_t)((rec_side<RB, 0>(f, xr) >> f.sb) & (uint32_t)(nd_ - 1));
-            }
+            const uint32_t r = tid + k * SORT_THREADS;
+            dr[k] = 0;
+            if (r < n) dr[k] = (rec_side<RB, 0>(f, take_rec<RB>(src, r)) >> f.sb) & (uint32_t)(nd_ - 1);
         }
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k)
-            if (threadIdx.x + k * SORT_THREADS < n) rk[k] = (uint16_t)atomicAdd(&hist[dg[k]], 1u);
+            if (tid + k * SORT_THREADS < n) dr[k] |= atomicAdd(&hist[dr[k]], 1u) << 16;
         __syncthreads();
-        const uint32_t n_tile = tile_scan_n(hist, dof, nd_, sh_scan);
-        for (int i = threadIdx.x; i < nd_; i += SORT_THREADS)
-            if (hist[i] && NN_IN(fb0 + i, B, p.status)) gbase[i] = atomicAdd(&p.gcur[fb0 + i], hist[i]);
+        // places of the digits, and the reserved global range of each present
+        // one (its atomic's answer is needed only after the placement below)
+        uint32_t gb[DPT];
+        {
+            const int i0 = tid * per;
+            uint32_t sum = 0;
+            if (i0 < nd_)
+                for (int i = 0; i < (DPT == 1 ? 1 : per); ++i) sum += hist[i0 + i];
+            uint32_t inc = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= d) inc += y;
+            }
+            if (lane == 31) sh_warp[warp] = inc;
+#pragma unroll
+            for (int i = 0; i < DPT; ++i) {
+                gb[i] = 0;
+                if (i < per && i0 < nd_) {
+                    const uint32_t h = hist[i0 + i];
+                    if (h && NN_IN(fb0 + i0 + i, B, p.status)) gb[i] = atomicAdd(&p.gcur[fb0 + i0 + i], h);
+                }
+            }
+            __syncthreads();
+            uint32_t run = inc - sum;
+            for (int w = 0; w < warp; ++w) run += sh_warp[w];
+            if (i0 < nd_)
+                for (int i = 0; i < (DPT == 1 ? 1 : per); ++i) {
+                    dof[i0 + i] = run;
+                    run += hist[i0 + i];
+                    hist[i0 + i] = 0;  // for the next tile
+                }
+        }
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k) {
-            if (rk[k] == 0xFFFF) continue;
-            const uint32_t q = dof[dg[k]] + rk[k];
-            if constexpr (FINE_RPT <= 4) put_rec<RB>(out, q, x[k]);
-            else put_rec<RB>(out, q, take_rec<RB>(src, threadIdx.x + k * SORT_THREADS));
-            odig[q] = dg[k];
+            const uint32_t r = tid + k * SORT_THREADS;
+            if (r < n) perm[dof[dr[k] & 0xffffu] + (dr[k] >> 16)] = (uint16_t)r;
         }
+#pragma unroll
+        for (int i = 0; i < DPT; ++i)
+            if (i < per && tid * per < nd_) delta[tid * per + i] = gb[i] - dof[tid * per + i];
         __syncthreads();
-        for (uint32_t q = threadIdx.x; q < n_tile; q += SORT_THREADS) {
-            const uint32_t dd = odig[q];
-            const uint64_t pos = (uint64_t)gbase[dd] + (q - dof[dd]);
-            if (pos < p.rec_cap) put_rec<RB>(p.rec, pos, take_rec<RB>(out, q));
+#pragma unroll
+        for (int k = 0; k < FINE_RPT; ++k) {
+            const uint32_t q = tid + k * SORT_THREADS;
+            if (q < n) {
+                const Rec x = take_rec<RB>(src, perm[q]);
+                const uint32_t pos = delta[(rec_side<RB, 0>(f, x) >> f.sb) & (uint32_t)(nd_ - 1)] + q;
+                if (pos < p.rec_cap) put_rec<RB>(p.rec, pos, x);
+            }
         }
-        __syncthreads();
+        // (no barrier: the next tile writes none of this before its first one)
     }
 }
 
 // Per bucket b: total records = sum over CTAs of hist[c][b]; bucket starts by
 // a lookback scan over tiles of buckets; each bucket's write cursor starts at
 // its start.
-__global__ void __launch_bounds__(OFFSETS_THREADS) k_offsets(OffsetsParams p) {
+// A tile has OFFSETS_THREADS buckets.  Its histogram rows (up to 304) are
+// shared out among the CTA's slices of that many threads: with one thread per
+// bucket the sum was a chain of loads, 22-34 us at any mesh size; now 12 us for 3,445 buckets, 16 us
+// for 16,384 and 27 us for 66,308 (23 before).  64 buckets and 16 slices took
+// 17 and 41 us for the last two.
+__global__ void __launch_bounds__(OFFSETS_THREADS * OFFSETS_SLICES) k_offsets(OffsetsParams p) {
+    __shared__ uint32_t sh_part[OFFSETS_SLICES][OFFSETS_THREADS];
     __shared__ uint64_t sh_scan[33];
     __shared__ uint32_t sh_tile;
     __shared__ uint64_t sh_base;
@@ -644,10 +668,20 @@ __global__ void __launch_bounds__(OFFSETS_THREADS) k_offsets(OffsetsParams p) {
     __syncthreads();
     const uint32_t tile = sh_tile;
     const int64_t B = p.hdr ? p.hdr->n_buckets : p.n_buckets;
-    const int64_t b = (int64_t)tile * blockDim.x + threadIdx.x;
+    const int col = threadIdx.x % OFFSETS_THREADS, slice = threadIdx.x / OFFSETS_THREADS;
+    const int slices = blockDim.x / OFFSETS_THREADS;
+    int64_t b = (int64_t)tile * OFFSETS_THREADS + col;
+    uint32_t sum = 0;
+    if (b < B) {
+#pragma unroll 10
+        for (int c = slice; c < p.n_cta; c += slices) sum += p.hist[(int64_t)c * B + b];
+    }
+    sh_part[slice][col] = sum;
+    __syncthreads();
+    if (slice) b = B;  // the first slice goes on, the others only take part in the barriers
     uint64_t tot = 0, nf = 0;
     if (b < B) {
-        for (int c = 0; c < p.n_cta; ++c) tot += p.hist[(int64_t)c * B + b];
+        for (int c = 0; c < slices; ++c) tot += sh_part[c][col];
         if (p.nfc) nf = p.nfc[b];
     }
     // records (low 31 bits) and repeated-node records (next 31) in one scan;
@@ -768,21 +802,40 @@ cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s) {
 
 // One CTA per resident slot (the SMs times the CTAs its shared memory
 // allows per SM): each CTA works through its tiles with the copies in flight.
-template <int RB, int RPT>
+template <int RB, int RPT, int DPT>
 cudaError_t fine_t(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
     const size_t fs = fine_smem(1 << p.fmt.cshift, RB);
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_part_fine<RB, RPT>, SORT_THREADS, fs);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_part_fine<RB, RPT, DPT>, SORT_THREADS, fs);
     if (e != cudaSuccess) return e;
-    k_part_fine<RB, RPT><<<std::max(1, sms * std::max(occ, 1)), SORT_THREADS, fs, s>>>(p, bstart);
+    k_part_fine<RB, RPT, DPT><<<std::max(1, sms * std::max(occ, 1)), SORT_THREADS, fs, s>>>(p, bstart);
     return cudaGetLastError();
+}
+
+template <int RB>
+cudaError_t fine_rb(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
+    const int nd = 1 << p.fmt.cshift;
+    if (nd < FINE_RPT_WIDE_DIGITS) return fine_t<RB, 4, FINE_RPT_WIDE_DIGITS / 2 / SORT_THREADS>(p, bstart, sms, s);
+    if (nd == FINE_RPT_WIDE_DIGITS) return fine_t<RB, 8, FINE_RPT_WIDE_DIGITS / SORT_THREADS>(p, bstart, sms, s);
+    return fine_t<RB, 8, FINE_DIGITS / SORT_THREADS>(p, bstart, sms, s);
 }
 
 cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
     if (p.fmt.cshift <= 0) return cudaSuccess;
-    const bool wide = fine_rpt(1 << p.fmt.cshift) == 8;
-    if (p.fmt.rb == 8) return wide ? fine_t<8, 8>(p, bstart, sms, s) : fine_t<8, 4>(p, bstart, sms, s);
-    return wide ? fine_t<16, 8>(p, bstart, sms, s) : fine_t<16, 4>(p, bstart, sms, s);
+    return p.fmt.rb == 8 ? fine_rb<8>(p, bstart, sms, s) : fine_rb<16>(p, bstart, sms, s);
+}
+
+template <int RB>
+cudaError_t set_fine_smem() {
+    cudaError_t e = cudaFuncSetAttribute(k_part_fine<RB, 4, FINE_RPT_WIDE_DIGITS / 2 / SORT_THREADS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_part_fine<RB, 8, FINE_RPT_WIDE_DIGITS / SORT_THREADS>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_part_fine<RB, 8, FINE_DIGITS / SORT_THREADS>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
+    return e;
 }
 
 cudaError_t launch_part_sorted(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
@@ -811,7 +864,7 @@ cudaError_t launch_slab_count(const EmitParams& p, int shift, int n_slabs, uint3
 cudaError_t launch_offsets(const OffsetsParams& p, cudaStream_t s) {
     const int64_t tiles = (p.n_buckets + OFFSETS_THREADS - 1) / OFFSETS_THREADS;
     if (tiles == 0) return cudaSuccess;
-    k_offsets<<<(unsigned)tiles, OFFSETS_THREADS, 0, s>>>(p);
+    k_offsets<<<(unsigned)tiles, OFFSETS_THREADS * (p.n_cta >= 16 ? OFFSETS_SLICES : 1), 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -821,14 +874,8 @@ cudaError_t set_emit_smem_all(size_t bytes) {
     if (e == cudaSuccess) e = set_sorted_smem<NN_TET>();
     if (e == cudaSuccess) e = set_sorted_smem<NN_HEX>();
     if (e == cudaSuccess) e = set_sorted_smem<NN_MIXED>();
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_part_fine<8, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_part_fine<8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_part_fine<16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_part_fine<16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
+    if (e == cudaSuccess) e = set_fine_smem<8>();
+    if (e == cudaSuccess) e = set_fine_smem<16>();
     if (e == cudaSuccess) e = set_emit_smem<NN_TRI>(bytes);
     if (e == cudaSuccess) e = set_emit_smem<NN_QUAD>(bytes);
     if (e == cudaSuccess) e = set_emit_smem<NN_TET>(bytes);

@@ -163,7 +163,8 @@ struct BucketParams {
 constexpr int EMIT_THREADS = 1024;
 constexpr int PART_THREADS = 512;
 constexpr int SORT_THREADS = 256;   // tile-sorted partition passes
-constexpr int OFFSETS_THREADS = 128;
+constexpr int OFFSETS_THREADS = 128;  // buckets per tile of the offsets scan
+constexpr int OFFSETS_SLICES = 8;     // slices of its histogram rows summed side by side
 constexpr int NODE_SCAN_TILE = 512;  // groups of 32 nodes per tile of the node-row placement's scan
 
 // Placement of the node rows the bucket pass left in scratch (nn_compact.cu).
