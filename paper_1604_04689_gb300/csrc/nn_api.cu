@@ -445,7 +445,7 @@ constexpr int BATCH_SLOTS = 24, BATCH_LIST = 256;
 struct BatchPlan {
     int sb = 7, groups = 4;
     int64_t B_cap = 0;
-    size_t hdr_bytes = 0, meshes_off = 0, elem_off_off = 0, bucket_off_off = 0, table_bytes = 0;
+    size_t hdr_bytes = 0, meshes_off = 0, elem_off_off = 0, bucket_off_off = 0, weight_off_off = 0, table_bytes = 0;
     size_t off_bcount = 0, off_bstart = 0, off_gcur = 0, off_rec = 0, off_lb_off = 0, off_ctrl = 0, off_spill = 0, ws_min = 0, ws_rec = 0, off_nfc = 0,
            off_estart = 0, off_ntmp = 0, off_grp = 0, off_nloc = 0, off_nstart = 0, off_lb_ns = 0;
     size_t bucket_smem = 0;
@@ -465,7 +465,8 @@ nn_status batch_plan(const nn_handle* h, const nn_batch_caps* c, BatchPlan* out)
     p.meshes_off = p.hdr_bytes;
     p.elem_off_off = p.meshes_off + align_up((size_t)c->max_meshes * sizeof(BatchMesh));
     p.bucket_off_off = p.elem_off_off + align_up(((size_t)c->max_meshes + 1) * 8);
-    p.table_bytes = p.bucket_off_off + align_up(((size_t)c->max_meshes + 1) * 8);
+    p.weight_off_off = p.bucket_off_off + align_up(((size_t)c->max_meshes + 1) * 8);
+    p.table_bytes = p.weight_off_off + align_up(((size_t)c->max_meshes + 1) * 8);
     // bucket kernel: the 24 slots of a tet mesh (a batch may hold any element
     // type), 128 threads for buckets of 128 nodes
     p.bucket_threads = 128;
@@ -497,7 +498,7 @@ nn_status batch_plan(const nn_handle* h, const nn_batch_caps* c, BatchPlan* out)
     p.off_spill = o;
     p.ws_min = o;
     p.ws_rec = o + (((size_t)16 << 20) + (size_t)c->max_conn * 8);
-    p.emit_grid = h->sms * (2048 / batch_threads());
+    p.emit_grid = h->sms * batch_ctas_per_sm();
     *out = p;
     return NN_OK;
 }
@@ -516,6 +517,7 @@ nn_status batch_prepare(nn_handle* h, const nn_batch_caps* c, const nn_mesh* mes
     BatchMesh* bm = reinterpret_cast<BatchMesh*>(sg + bp.meshes_off);
     int64_t* eoff = reinterpret_cast<int64_t*>(sg + bp.elem_off_off);
     int64_t* boff = reinterpret_cast<int64_t*>(sg + bp.bucket_off_off);
+    int64_t* woff = reinterpret_cast<int64_t*>(sg + bp.weight_off_off);
     int64_t E = 0, Bk = 0, C = 0, Nn = 0, maxT = 0, maxN = 0;
     for (int m = 0; m < n; ++m) {
         const nn_mesh& M = meshes[m];
@@ -543,6 +545,7 @@ nn_status batch_prepare(nn_handle* h, const nn_batch_caps* c, const nn_mesh* mes
         d.status = d_status + m;
         eoff[m] = E;
         boff[m] = Bk;
+        woff[m] = C + E;
         E += M.n_elems;
         Bk += (M.n_nodes + (1ll << bp.sb) - 1) >> bp.sb;
         C += M.n_conn;
@@ -552,6 +555,7 @@ nn_status batch_prepare(nn_handle* h, const nn_batch_caps* c, const nn_mesh* mes
     }
     eoff[n] = E;
     boff[n] = Bk;
+    woff[n] = C + E;
     if (E > c->max_elems || C > c->max_conn || Nn > c->max_nodes || Bk > bp.B_cap) return NN_ERR_BUDGET;
     RecFmt f{};
     if (!record_format(bp.sb, c->want, 3, maxT, maxN, -1, 16, &f)) return NN_ERR_ARG;
@@ -578,6 +582,7 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     bt.meshes = reinterpret_cast<const BatchMesh*>(w + bp.meshes_off);
     bt.elem_off = reinterpret_cast<const int64_t*>(w + bp.elem_off_off);
     bt.bucket_off = reinterpret_cast<const int64_t*>(w + bp.bucket_off_off);
+    bt.weight_off = reinterpret_cast<const int64_t*>(w + bp.weight_off_off);
     uint32_t* bcount = reinterpret_cast<uint32_t*>(w + bp.off_bcount);
     uint32_t* nfc = reinterpret_cast<uint32_t*>(w + bp.off_nfc);
     uint32_t* gcur = reinterpret_cast<uint32_t*>(w + bp.off_gcur);

@@ -98,8 +98,8 @@ struct OffsetsParams {
 // A batch is the disjoint union of many meshes built by one launch sequence.
 // Its description lives in device memory (copied from host staging by the
 // launch), so the same captured sequence serves any batch that fits the
-// workspace capacity: header, then one BatchMesh per mesh, then the element
-// and bucket offsets of the meshes (n_meshes + 1 each).
+// workspace capacity: header, then one BatchMesh per mesh, then the element,
+// bucket and weight offsets of the meshes (n_meshes + 1 each).
 struct BatchMesh {
     int32_t type;
     int32_t k;
@@ -125,6 +125,7 @@ struct BatchTables {
     const BatchMesh* meshes;
     const int64_t* elem_off;    // [n_meshes+1]
     const int64_t* bucket_off;  // [n_meshes+1]
+    const int64_t* weight_off;  // [n_meshes+1] incidences and elements of the meshes before
 };
 
 // Bucket pass: one CTA per bucket (persistent, buckets taken in order),
@@ -229,7 +230,7 @@ cudaError_t bucket_occupancy(int* blocks, int threads, int imax, size_t smem);
 cudaError_t launch_batch_emit(const BatchTables& bt, uint32_t* bcount, uint32_t* nfc, uint32_t* gcur, uint8_t* rec,
                               uint64_t* lb_off, uint32_t* ctrl, int grid, int stage, cudaStream_t s,
                               uint64_t* lb_ns = nullptr);
-int batch_threads();
+int batch_ctas_per_sm();
 cudaError_t set_emit_smem_all(size_t bytes);
 cudaError_t set_bucket_smem_all(size_t bytes);
 bool handle_offline(const nn_handle* h);  // a sizing-only handle (nn_create_offline)

@@ -223,3 +223,16 @@ def test_one_call_submit_refuses_a_capturing_stream():
         assert all(int(rp[0].item()) == -3 for rp, _ in outs)
     finally:
         nn.nn_destroy(h)
+
+
+@pytest.mark.parametrize("sb", [4, 7])
+def test_slices_with_and_without_shared_counters(sb):
+    # buckets of 16 nodes: the middle mesh has more of them (10,000) than a
+    # CTA's shared counters (8,192), its neighbours' slices reach into it or
+    # not; buckets of 128 nodes: every slice counts in shared memory
+    meshes = [mg.tri_grid(3, 1), mg.hex_grid(20, 2), mg.tri_grid(400, 3), mg.mixed_grid(9, 4), mg.tet_grid(12, 5),
+              mg.Mesh(mg.TRI, 0, np.zeros(0, np.int32)), mg.Mesh(mg.HEX, 9, np.zeros(0, np.int32))]
+    bb = nn.BatchBuilder(**caps_for(meshes), sb=sb)
+    for order in (meshes, meshes[::-1]):
+        for r, m in zip(bb.run([nn.DeviceMesh.from_host(m) for m in order]), order):
+            check(r, m)
