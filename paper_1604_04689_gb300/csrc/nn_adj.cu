@@ -19,8 +19,9 @@
 // element, and every element of a mixed mesh, merges the (sorted) element
 // rows of its distinct nodes, which yields every element sharing a node with
 // it once, in ascending order, with the number of shared nodes; the face
-// tests run only where that number allows a shared face.  Then count,
-// exclusive scan (decoupled lookback over tiles of elements), and write.
+// tests run only where that number allows a shared face.  Their counts come
+// first, then one pass scans all counts (decoupled lookback over tiles of
+// elements) and writes the matched rows, then the merged rows are written.
 #include "nn_device.cuh"
 
 namespace nn {
@@ -28,7 +29,7 @@ namespace nn {
 namespace {
 
 constexpr int ADJ_THREADS = 256;
-constexpr int ADJ_SCAN_THREADS = 128;
+constexpr int ADJ_TILE = 1024;  // elements of a tile of the row pass
 
 __constant__ int8_t c_nfaces[4] = {3, 4, 4, 6};
 __constant__ int8_t c_fsize[4] = {2, 2, 3, 4};
@@ -136,9 +137,17 @@ __device__ __forceinline__ void for_each_neighbour(const AdjParams& p, int64_t e
 // of 32 lanes were active on average, and every element's node rows were
 // walked twice.  Matching per node gathers each element's nodes once per node
 // (n_conn gathers in all) and has no data-dependent branch but the rare match.
-// Whole call, GB300: 101^3 Kuhn grid 26.7 -> 1.7 ms, 161^3 111 -> 6.9 ms,
-// 129^3 hex grid 3.0 -> 0.94 ms, 2048^2 triangle grid 7.3 -> 1.4 ms.  The
-// groups have 8 lanes where a node has 4 to 8 elements, a warp for tets (24).
+// Whole call, GB300: 101^3 Kuhn grid 26.7 -> 1.8 ms, and 0.98 ms with the
+// face table and the one-pass rows below; 129^3 hex grid 3.0 -> 0.94 ms and
+// 2048^2 triangle grid 7.3 -> 1.4 ms before the latter.  The groups have 8 lanes where a node has 4 to 8 elements, a warp for tets (24).
+//
+// Tets: comparing each of a node's 24 elements with the 23 others was bound by
+// instructions (78 % of issue slots).  A face needs a look only at its
+// smallest node, by a third of its elements' faces there, and two tets share a
+// face exactly when its three nodes are equal: the faces go into a small hash
+// table per warp.  Hexes and quads also ask whether a face's nodes lie in an
+// element whose face it is not, and compare pairs in groups of 8.
+constexpr int FACE_HASH_BITS = 7;
 constexpr int ADJ_LONG = 64;  // longest node row matched here; elements around a longer one are flagged
 
 template <int TYPE>
@@ -291,6 +300,8 @@ template <int TYPE>
 __global__ void __launch_bounds__(ADJ_THREADS) k_adj_match(AdjParams p) {
     using S = AdjShape<TYPE>;
     constexpr int G = S::G, PER = 32 / G;
+    __shared__ __align__(16) uint32_t sh_head[TYPE == NN_TET ? ADJ_THREADS / 32 : 1][1 << FACE_HASH_BITS];
+    __shared__ uint4 sh_face[TYPE == NN_TET ? ADJ_THREADS / 32 : 1][32 * S::F];
     const int lane = threadIdx.x & 31, gl = lane & (G - 1);
     const int64_t warp = ((int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x) >> 5;
     const int64_t step = ((int64_t)gridDim.x * ADJ_THREADS >> 5) * PER;
@@ -327,13 +338,21 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_match(AdjParams p) {
             n = __ldg(p.ne_rp + v + 1) - a;
         }
     };
-    int64_t r0, L;
+    auto around = [&](int64_t a, int64_t n) { return n <= G && gl < n ? __ldg(p.ne_col + a + gl) : -1; };
+    // the next node's elements and the bounds of the one after it are on their
+    // way while a node's elements are compared
+    int64_t r0, L, r1, L1;
     row(base, r0, L);
+    row(base + step, r1, L1);
+    int32_t e0 = around(r0, L);
     for (; base < p.n_nodes; base += step) {
         const int32_t v = (int32_t)(base + lane / G);
         const int64_t cur = r0, n = L;
-        const int32_t e = n <= G && gl < n ? __ldg(p.ne_col + cur + gl) : -1;
-        row(base + step, r0, L);  // the next node's row, while this one's elements are on their way
+        const int32_t e = e0;
+        r0 = r1;
+        L = L1;
+        e0 = around(r0, L);
+        row(base + 2 * step, r1, L1);
         AdjFrame<TYPE> x{};
         const int ok = x.load(p, e, v);
         const int32_t id = ok ? e : -1;
@@ -343,13 +362,51 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_match(AdjParams p) {
             if ((m & (G == 32 ? 0xffffffffu : (1u << (G & 31)) - 1)) && ok) p.cplx[e] = 1;
         }
         Found r{};
-        const int jmax = (int)__reduce_max_sync(0xffffffffu, n <= G && n > 1 ? (unsigned)n : 0u);
-        for (int j = 0; j < jmax; ++j) {
-            const int32_t ey = __shfl_sync(0xffffffffu, id, j, G);
-            int32_t y[S::Q];
+        if constexpr (TYPE == NN_TET) {
+            // the faces at v whose smallest node v is, by their other two
+            // nodes: chained by hash, and each compared with its chain
+            if (n > 1 && n <= G) {
+                uint32_t* const head = sh_head[threadIdx.x >> 5];
+                uint4* const face = sh_face[threadIdx.x >> 5];
+                reinterpret_cast<uint4*>(head)[lane] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+                __syncwarp();
+                uint32_t a[S::F], b[S::F], h[S::F];
+                bool use[S::F];
 #pragma unroll
-            for (int k = 0; k < S::Q; ++k) y[k] = __shfl_sync(0xffffffffu, x.q[k], j, G);
-            if (ok && ey >= 0 && ey != e) compare(x, v, ey, y, r);
+                for (int f = 0; f < S::F; ++f) {
+                    const int32_t s = x.q[f == 0 ? 1 : 0], t = x.q[f == 2 ? 1 : 2];
+                    use[f] = ok == 1 && s > v && t > v;
+                    a[f] = (uint32_t)min(s, t);
+                    b[f] = (uint32_t)max(s, t);
+                    h[f] = (a[f] * 0x9E3779B1u + b[f] * 0x85EBCA6Bu) >> (32 - FACE_HASH_BITS);
+                    if (use[f]) {
+                        const uint32_t next = atomicExch(&head[h[f]], (uint32_t)(f * 32 + lane));
+                        face[f * 32 + lane] = make_uint4(a[f], b[f], (uint32_t)e, next);
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int f = 0; f < S::F; ++f) {
+                    for (uint32_t k = use[f] ? head[h[f]] : EMPTY; k != EMPTY;) {
+                        const uint4 y = face[k];
+                        if (y.x == a[f] && y.y == b[f] && y.z != (uint32_t)e) {
+                            r.y[f] = (int32_t)y.z;
+                            ++r.n[f];
+                        }
+                        k = y.w;
+                    }
+                }
+                __syncwarp();
+            }
+        } else {
+            const int jmax = (int)__reduce_max_sync(0xffffffffu, n <= G && n > 1 ? (unsigned)n : 0u);
+            for (int j = 0; j < jmax; ++j) {
+                const int32_t ey = __shfl_sync(0xffffffffu, id, j, G);
+                int32_t y[S::Q];
+#pragma unroll
+                for (int k = 0; k < S::Q; ++k) y[k] = __shfl_sync(0xffffffffu, x.q[k], j, G);
+                if (ok && ey >= 0 && ey != e) compare(x, v, ey, y, r);
+            }
         }
         if (ok == 1) settle(x, v, e, r);
         if (n <= G) continue;
@@ -396,107 +453,152 @@ __device__ __forceinline__ void sorted_slots(const AdjParams& p, int64_t e, uint
         }
 }
 
-// NF: slots per element (0: no slots, every element merges its node rows).
-template <int NF>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_count(AdjParams p) {
-    for (int64_t e = (int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x; e < p.n_elems;
-         e += (int64_t)gridDim.x * ADJ_THREADS) {
-        uint32_t c = 0;
-        bool slow = true;
-        if constexpr (NF > 0) {
-            slow = p.cplx[e];
-            if (!slow) {
-                int32_t nd[8];
-                const int t = load_element(p, e, nd);
-                if (t >= 0) {  // (an invalid element is in no node's row: its slots were never written)
-                    uint32_t s[NF];
-                    sorted_slots<NF>(p, e, s);
+// Whether element e (of type TYPE) has all its nodes in range.  An element
+// that has not is in no node's row, and its slots were never written.
+template <int TYPE>
+__device__ __forceinline__ bool valid_element(const AdjParams& p, int64_t e) {
+    constexpr int NPE = AdjShape<TYPE>::Q + 1;
+    const uint32_t N = (uint32_t)p.n_nodes;  // below 2^31
+    if constexpr (NPE == 3) {
+        bool ok = true;
 #pragma unroll
-                    for (int i = 0; i < NF; ++i) c += s[i] != EMPTY && (i == 0 || s[i] != s[i - 1]);
-                }
-            }
+        for (int i = 0; i < 3; ++i) ok = ok && (uint32_t)__ldg(p.conn + 3 * e + i) < N;
+        return ok;
+    } else {
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < NPE / 4; ++q) {
+            const uint4 a = __ldg(reinterpret_cast<const uint4*>(p.conn) + (NPE / 4) * e + q);
+            ok = ok && a.x < N && a.y < N && a.z < N && a.w < N;
         }
-        if (slow) for_each_neighbour(p, e, [&](int32_t) { ++c; });
-        p.cnt[e] = c;
+        return ok;
     }
 }
 
-__global__ void __launch_bounds__(ADJ_SCAN_THREADS) k_adj_scan(AdjParams p) {
+__device__ __noinline__ uint32_t merge_count(const AdjParams& p, int64_t e) {
+    uint32_t c = 0;
+    for_each_neighbour(p, e, [&](int32_t) { ++c; });
+    return c;
+}
+__device__ __noinline__ void merge_write(const AdjParams& p, int64_t e, int32_t* row, int64_t n) {
+    int64_t k = 0;
+    for_each_neighbour(p, e, [&](int32_t f) {
+        if (k < n) row[k] = f;
+        ++k;
+    });
+}
+
+// Elements whose rows are merged from their nodes' rows: the flagged ones,
+// or all (a mixed mesh, or no room for the slots).  Their counts, before the
+// offsets are known, and their rows, after.  (They are not part of the pass
+// between: a merge may take long, and no tile of the scan waits for one.)
+template <bool WRITE>
+__global__ void __launch_bounds__(ADJ_THREADS) k_adj_merge(AdjParams p) {
+    for (int64_t e = (int64_t)blockIdx.x * ADJ_THREADS + threadIdx.x; e < p.n_elems;
+         e += (int64_t)gridDim.x * ADJ_THREADS) {
+        if (p.nbr && !p.cplx[e]) continue;
+        if constexpr (WRITE) {
+            const int64_t a = p.rp[e], n = p.rp[e + 1] - a;
+            if (n > 0 && a + n <= p.cap) merge_write(p, e, p.col + a, n);
+        } else {
+            p.cnt[e] = merge_count(p, e);
+        }
+    }
+}
+
+// Row pointers of all elements and the rows of the matched ones, in one pass:
+// a tile's rows are put together in shared memory and written as one run at
+// the offset that the lookback over the earlier tiles gives.  (Counting,
+// scanning and writing in a kernel each read the slots twice and ran 47,000
+// tiles of 128 elements for 6 M of them.)  TYPE = NN_MIXED: no slots, the
+// counts are scanned alone.
+constexpr int ROWS_PER = ADJ_TILE / ADJ_THREADS;  // elements of a thread
+template <int TYPE>
+__global__ void __launch_bounds__(ADJ_THREADS) k_adj_rows(AdjParams p) {
+    constexpr int NF = TYPE == NN_MIXED ? 0 : AdjShape<TYPE == NN_MIXED ? NN_TET : TYPE>::NF;
+    __shared__ uint32_t rows[NF > 0 ? ADJ_TILE * NF : 1];
     __shared__ uint64_t sh_scan[33];
     __shared__ uint32_t sh_tile;
     __shared__ uint64_t sh_base;
     if (threadIdx.x == 0) sh_tile = atomicAdd(p.ticket, 1u);
     __syncthreads();
     const uint32_t tile = sh_tile;
-    const int64_t e = (int64_t)tile * ADJ_SCAN_THREADS + threadIdx.x;
-    const uint64_t x = e < p.n_elems ? p.cnt[e] : 0;
+    const int64_t e0 = (int64_t)tile * ADJ_TILE + threadIdx.x * ROWS_PER;
+    uint32_t s[ROWS_PER][NF > 0 ? NF : 1];
+    uint32_t n[ROWS_PER];
+    bool slow[ROWS_PER];
+    uint64_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < ROWS_PER; ++k) {
+        const int64_t e = e0 + k;
+        n[k] = 0;
+        slow[k] = true;
+        if (e < p.n_elems) {
+            if constexpr (NF > 0) {
+                slow[k] = p.cplx[e];
+                if (!slow[k] && valid_element<TYPE>(p, e)) {
+                    sorted_slots<NF>(p, e, s[k]);
+#pragma unroll
+                    for (int i = 0; i < NF; ++i) n[k] += s[k][i] != EMPTY && (i == 0 || s[k][i] != s[k][i - 1]);
+                }
+            }
+            if (slow[k]) n[k] = p.cnt[e];
+        }
+        sum += n[k];
+    }
     uint64_t agg;
-    const uint64_t ex = block_excl_scan(x, &agg, sh_scan);
+    const uint64_t ex = block_excl_scan(sum, &agg, sh_scan);
     if (threadIdx.x < 32) {
         const uint64_t base = warp_lookback(p.lb_state, tile, agg, p.status);
         if (threadIdx.x == 0) sh_base = base;
     }
-    __syncthreads();
-    if (e < p.n_elems) p.rp[e] = (int64_t)(sh_base + ex);
-    if (e == p.n_elems - 1) {
-        p.rp[p.n_elems] = (int64_t)(sh_base + ex + x);
-        if ((int64_t)(sh_base + ex + x) > p.cap) set_status(p.status, NN_ERR_CAPACITY);
-    }
-}
-
-template <int NF>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_write(AdjParams p) {
-    // the rows of a block's elements follow one another: put together in
-    // shared memory and written as one run
-    __shared__ uint32_t rows[NF > 0 ? ADJ_THREADS * NF : 1];
-    for (int64_t e0 = (int64_t)blockIdx.x * ADJ_THREADS; e0 < p.n_elems; e0 += (int64_t)gridDim.x * ADJ_THREADS) {
-        const int64_t e = e0 + threadIdx.x;
-        const int64_t a = e < p.n_elems ? p.rp[e] : 0, n = e < p.n_elems ? p.rp[e + 1] - a : 0;
-        bool slow = n > 0;
-        if constexpr (NF > 0) {
-            slow = n > 0 && p.cplx[e];
-            if (!__syncthreads_or(slow)) {
-                const int64_t a0 = p.rp[e0], a1 = p.rp[min(e0 + ADJ_THREADS, p.n_elems)];
-                if (n > 0) {
-                    uint32_t s[NF];
-                    sorted_slots<NF>(p, e, s);
-                    uint32_t* d = rows + (a - a0);
+    if constexpr (NF > 0) {
+        // (a tile of merged elements alone may have longer rows than this holds; theirs are left out here)
+        if (agg <= ADJ_TILE * NF) {
+            uint32_t* d = rows + ex;
 #pragma unroll
-                    for (int i = 0; i < NF; ++i)
-                        if (s[i] != EMPTY && (i == 0 || s[i] != s[i - 1])) *d++ = s[i];
+            for (int k = 0; k < ROWS_PER; ++k) {
+                if (slow[k]) {
+                    d += n[k];
+                    continue;
                 }
-                __syncthreads();
-                if (a1 <= p.cap)
-                    for (int64_t i = threadIdx.x; i < a1 - a0; i += ADJ_THREADS) p.col[a0 + i] = (int32_t)rows[i];
-                __syncthreads();
-                continue;
-            }
-            if (n > 0 && !slow && a + n <= p.cap) {
-                uint32_t s[NF];
-                sorted_slots<NF>(p, e, s);
-                int32_t* d = p.col + a;
 #pragma unroll
                 for (int i = 0; i < NF; ++i)
-                    if (s[i] != EMPTY && (i == 0 || s[i] != s[i - 1])) *d++ = (int32_t)s[i];
+                    if (n[k] && s[k][i] != EMPTY && (i == 0 || s[k][i] != s[k][i - 1])) *d++ = s[k][i];
             }
         }
-        if (slow && a + n <= p.cap) {
-            int32_t* row = p.col + a;
-            int64_t k = 0;
-            for_each_neighbour(p, e, [&](int32_t f) {
-                if (k < n) row[k] = f;
-                ++k;
-            });
+    }
+    __syncthreads();
+    const uint64_t base = sh_base;
+    uint64_t at = base + ex;
+#pragma unroll
+    for (int k = 0; k < ROWS_PER; ++k) {
+        if (e0 + k < p.n_elems) p.rp[e0 + k] = (int64_t)at;
+        if constexpr (NF > 0) {
+            if (agg > ADJ_TILE * NF && !slow[k] && at + n[k] <= (uint64_t)p.cap) {
+                int32_t* d = p.col + at;
+#pragma unroll
+                for (int i = 0; i < NF; ++i)
+                    if (n[k] && s[k][i] != EMPTY && (i == 0 || s[k][i] != s[k][i - 1])) *d++ = (int32_t)s[k][i];
+            }
         }
+        at += n[k];
+        if (e0 + k == p.n_elems - 1) {
+            p.rp[p.n_elems] = (int64_t)at;
+            if (at > (uint64_t)p.cap) set_status(p.status, NN_ERR_CAPACITY);
+        }
+    }
+    if constexpr (NF > 0) {
+        if (agg <= ADJ_TILE * NF && base + agg <= (uint64_t)p.cap)
+            for (uint32_t i = threadIdx.x; i < (uint32_t)agg; i += ADJ_THREADS) p.col[base + i] = (int32_t)rows[i];
     }
 }
 
-template <int NF>
+template <int TYPE>
 void count_scan_write(const AdjParams& p, int grid, cudaStream_t s) {
-    k_adj_count<NF><<<grid, ADJ_THREADS, 0, s>>>(p);
-    const unsigned tiles = (unsigned)((p.n_elems + ADJ_SCAN_THREADS - 1) / ADJ_SCAN_THREADS);
-    k_adj_scan<<<tiles, ADJ_SCAN_THREADS, 0, s>>>(p);
-    k_adj_write<NF><<<grid, ADJ_THREADS, 0, s>>>(p);
+    k_adj_merge<false><<<grid, ADJ_THREADS, 0, s>>>(p);
+    k_adj_rows<TYPE><<<(unsigned)((p.n_elems + ADJ_TILE - 1) / ADJ_TILE), ADJ_THREADS, 0, s>>>(p);
+    k_adj_merge<true><<<grid, ADJ_THREADS, 0, s>>>(p);
 }
 
 template <int TYPE>
@@ -504,7 +606,7 @@ void match_and_write(const AdjParams& p, int grid, int sms, cudaStream_t s) {
     constexpr int NODES = ADJ_THREADS / AdjShape<TYPE>::G;  // nodes of a CTA at a time
     const int64_t blocks = (p.n_nodes + NODES - 1) / NODES;
     k_adj_match<TYPE><<<(unsigned)(blocks < (int64_t)sms * 16 ? blocks : (int64_t)sms * 16), ADJ_THREADS, 0, s>>>(p);
-    count_scan_write<AdjShape<TYPE>::NF>(p, grid, s);
+    count_scan_write<TYPE>(p, grid, s);
 }
 
 }  // namespace
@@ -518,7 +620,7 @@ int adjacency_slots(int type) {
 cudaError_t launch_adjacency(const AdjParams& p, int grid, int sms, cudaStream_t s) {
     if (p.n_elems <= 0) return cudaSuccess;
     if (!p.nbr) {
-        count_scan_write<0>(p, grid, s);
+        count_scan_write<NN_MIXED>(p, grid, s);
         return cudaGetLastError();
     }
     switch (p.type) {
@@ -530,6 +632,6 @@ cudaError_t launch_adjacency(const AdjParams& p, int grid, int sms, cudaStream_t
     return cudaGetLastError();
 }
 
-size_t adjacency_scan_tiles(int64_t n_elems) { return (size_t)((n_elems + ADJ_SCAN_THREADS - 1) / ADJ_SCAN_THREADS); }
+size_t adjacency_scan_tiles(int64_t n_elems) { return (size_t)((n_elems + ADJ_TILE - 1) / ADJ_TILE); }
 
 }  // namespace nn

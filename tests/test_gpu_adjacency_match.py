@@ -75,3 +75,17 @@ def test_boundary_cases_of_the_grids():
         ref = oracle.element_adjacency(mesh)["adj"]
         np.testing.assert_array_equal(rp.cpu().numpy(), ref[0])
         np.testing.assert_array_equal(col.cpu().numpy(), ref[1])
+
+
+@pytest.mark.parametrize("T", [1, 255, 1023, 1024, 1025, 2049])
+def test_row_pass_tile_edges(T):
+    # element counts around the row pass's tiles (1024 elements), every type
+    for grid in (mg.tri_grid(41, 3), mg.quad_grid(60, 4), mg.tet_grid(9, 5), mg.hex_grid(15, 6)):
+        mesh = mg.Mesh(grid.etype, grid.n_nodes, grid.conn[: T * mg.NPE[grid.etype]].copy())
+        assert mesh.n_elems == T
+        b = nn.Builder()
+        dm = nn.DeviceMesh.from_host(mesh)
+        rp, col = b.element_neighbors(dm, b.build(dm, nn.WANT_ELEMS)["elems"])
+        ref = oracle.element_adjacency(mesh)["adj"]
+        np.testing.assert_array_equal(rp.cpu().numpy(), ref[0])
+        np.testing.assert_array_equal(col.cpu().numpy(), ref[1])
