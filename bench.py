@@ -1007,7 +1007,7 @@ def time_adjacency(torch, nn, b, dm, out, flush, stream, steps):
     assert int(b.status.item()) == 0
     ms = sorted(times)[len(times) // 2]
     return {"ms_median": ms, "melem_per_s": dm.n_elems / (ms * 1e-3) / 1e6, "nnz": int(col.numel()),
-            "gpu_launches_per_call": 3, "steps": steps}
+            "gpu_launches_per_call": 3 if dm.etype == nn.MIXED else 4, "steps": steps}
 
 
 def max_over_ranks(x, world, device):
@@ -1028,16 +1028,19 @@ def whole_job_value(n_elems, steps, world, total_ms):
 
 
 def launches_per_build(plan, want="both"):
-    """Kernels one build launches: histogram, offsets, partition (one pass, or
-    coarse + fine when the buckets span more than 256 coarse digits), bucket,
-    and for node rows their placement (scan + copy)."""
+    """Kernels one build launches, from its plan; of a plan that does not say:
+    histogram, offsets, partition (one pass, or coarse + fine when the buckets
+    span more than 256 coarse digits), bucket, and for node rows their
+    placement (scan + copy)."""
+    if "kernels" in plan:
+        return plan["kernels"]
     return 3 + (2 if plan["partition"] > 0 else 1) + (2 if want in ("both", "nodes") else 0)
 
 
 # the sources that compile the single-mesh build's kernels and their launch
 # plan: traffic counters taken on other sources no longer describe them
 MEASURED_SOURCES = ("nn_api.cu", "nn_bucket.cu", "nn_bucket.cuh", "nn_bucket16.cu",
-                    "nn_bucket32.cu", "nn_bulk.cuh", "nn_compact.cu", "nn_device.cuh", "nn_emit.cu",
+                    "nn_bucket32.cu", "nn_bucket_direct.cu", "nn_bucket_direct32.cu", "nn_bulk.cuh", "nn_compact.cu", "nn_device.cuh", "nn_emit.cu",
                     "nn_internal.h")
 
 

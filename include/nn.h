@@ -155,7 +155,9 @@ nn_status nn_element_neighbors(nn_handle* h, const nn_mesh* mesh, const nn_csr* 
  * element walk, [3] bytes per incidence record, [4] minimum workspace bytes,
  * [5] CTAs of the bucket pass, [6] threads per bucket CTA, [7] shared memory
  * per bucket CTA, [8] partition mode (-1 scattered, 0 one sorted pass, k > 0
- * coarse + fine sorted passes with 2^k buckets per coarse region). */
+ * coarse + fine sorted passes with 2^k buckets per coarse region; the mode of
+ * a partitioned build: small meshes are built without), [9] kernels one build
+ * launches. */
 nn_status nn_plan_info(nn_handle* h, const nn_mesh* mesh, int want, int64_t* info, int n);
 
 /* Neighbor nodes of every node (Sec. 2.1.1, Sec. 2.2.1) into *out. */

@@ -21,7 +21,7 @@ struct nn_handle {
     size_t bucket_smem = 0;    // largest dynamic shared memory of the bucket kernel
     size_t smem_per_sm = 0;
     int sb_override = -1;      // fixed bucket width (tests / tuning), -1 = automatic
-    int part_mode = -1;        // -1 automatic, 0 one scattered store per record (tests)
+    int part_mode = -1;        // -1 automatic, 0 one scattered store per record, 1 always partitioned (tests)
     int64_t hist_chunk_override = 0;  // > 0: count at most this many buckets per walk (tests)
     int emit_ctas_override = 0;       // > 0: at most this many element-walk CTAs (tests)
     nn_tuning tuning{};        // nn_set_tuning: bucket width, block size, CTAs per SM (0 = automatic)
@@ -41,6 +41,8 @@ using namespace nn;
 
 constexpr size_t ALIGN = 256;
 constexpr int SB_MIN = 4, SB_MAX = 11;
+constexpr int64_t DIRECT_CONN = 1 << 16;  // incidences up to which a mesh is built without a partition (mixed: half)
+constexpr int DIRECT_QUEUE = 16384;       // incidences a direct build's CTA queues at a time (64 KB)
 
 size_t align_up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 int bits_for(uint64_t x) {  // bits needed to hold values 0..x (>= 1)
@@ -70,6 +72,8 @@ struct Plan {
     int bucket_threads = 256;
     int imax = 32, slots = 8, list_cap = 32;  // bucket pass: variant, places per node, listed records
     int groups = 1;                           // groups of 32 nodes per bucket
+    bool direct = false;                      // no partition: every bucket's CTA reads the whole connectivity
+    int queue_cap = 0;                        // ... incidences it queues at a time
     size_t bucket_smem = 0;
 };
 
@@ -149,6 +153,19 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     auto need = [&](int s, int slots) { return bucket_smem_bytes(s, want, p.k, slots, 16, list_of(s)); };
     p.bucket_threads = h->tuning.bucket_threads ? h->tuning.bucket_threads
                        : (need(8, want_slots) <= h->smem_per_sm / 2 - 2048 ? 256 : 128);
+    // A small mesh is built without a partition (nn_bucket.cuh, direct
+    // builds), one bucket per SM at most: histogram, offsets and partition are
+    // three launches with little to do, while reading the connectivity in
+    // every bucket's CTA grows with it.  Graph replays, direct and
+    // partitioned: triangles 3 K incidences 16 and 27 us, 24 K 19 and 30,
+    // quads 16 K 16 and 23, tets 12 K 27 and 35, 41 K 33 and 35, 81 K 38 and
+    // 35, hexes 64 K 27 and 31, mixed 22 K 33 and 37, 43 K 44 and 41; with
+    // more buckets than SMs a second wave doubles the time.
+    const bool tuned = h->sb_override >= 0 || h->part_mode >= 0 || h->hist_chunk_override > 0 ||
+                       h->emit_ctas_override > 0 || h->tuning.bucket_ctas_per_sm;
+    // (more elements than incidences: an invalid elem_ptr, left to the general path)
+    const bool direct = !tuned && lo == 0 && span == m->n_nodes && p.n_conn > 0 && p.T <= p.n_conn &&
+                        p.n_conn <= (p.type == NN_MIXED ? DIRECT_CONN / 2 : DIRECT_CONN);
     const int64_t B_max = (int64_t)1 << 20;  // (bounds the workspace tables)
     int sb = p.bucket_threads == 128 ? 7 : 8;
     if (h->tuning.bucket_ctas_per_sm) {  // the widest bucket that leaves room for that many CTAs
@@ -157,7 +174,7 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
         while (sb > SB_MIN && need(sb, want_slots) > budget) --sb;
     } else {
         // a small mesh: buckets for every SM, as long as one partition pass (256 buckets) does
-        while (sb > 5 && nbk(sb) < 2 * (int64_t)h->sms && nbk(sb - 1) <= 256) --sb;
+        while (sb > 5 && nbk(sb) < 2 * (int64_t)h->sms && nbk(sb - 1) <= (direct ? h->sms : 256)) --sb;
     }
     if (h->tuning.sb >= SB_MIN && h->tuning.sb <= SB_MAX) sb = h->tuning.sb;
     if (h->sb_override >= SB_MIN && h->sb_override <= SB_MAX) sb = h->sb_override;
@@ -202,6 +219,11 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     if (h->offline || bucket_occupancy(&per_sm, p.bucket_threads, p.imax, p.bucket_smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     p.bucket_grid = (int)std::min<int64_t>(p.B, (int64_t)h->sms * per_sm);
+
+    if (direct && f.cshift == 0 && p.B <= h->sms && p.bucket_smem + DIRECT_QUEUE * 4 <= h->bucket_smem) {
+        p.direct = true;
+        p.queue_cap = DIRECT_QUEUE;
+    }
 
     // workspace layout
     size_t o = 0;
@@ -296,8 +318,8 @@ nn_status run(nn_handle* h, const nn_mesh* m, int want, nn_csr* nodes, nn_csr* e
     uint8_t* w = static_cast<uint8_t*>(ws);
     if (h->prof) prof_flush(h);
     prof_mark(h, 0, s);
-    if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return NN_ERR_CUDA;
     if (p.N == 0) {
+        if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess) return NN_ERR_CUDA;
         if ((want & NN_WANT_NODES) && cudaMemsetAsync(nodes->row_ptr, 0, 8, s) != cudaSuccess) return NN_ERR_CUDA;
         if ((want & NN_WANT_ELEMS) && cudaMemsetAsync(elems->row_ptr, 0, 8, s) != cudaSuccess) return NN_ERR_CUDA;
         return NN_OK;
@@ -316,7 +338,11 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     auto mark = [&](int i) {
         if (prof) prof_mark(h, i, s);
     };
-    if (cudaMemsetAsync(w + p.zero_begin, 0, p.zero_end - p.zero_begin, s) != cudaSuccess) return NN_ERR_CUDA;
+    const size_t zero = p.direct ? p.off_ctrl : p.zero_begin;
+    // (the chunks of a chunked build keep one status word)
+    if ((base ? cudaMemsetAsync(w + zero, 0, p.zero_end - zero, s)
+              : launch_init(w + zero, p.zero_end - zero, d_status, h->sms, s)) != cudaSuccess)
+        return NN_ERR_CUDA;
 
     uint32_t* ctrl = reinterpret_cast<uint32_t*>(w + p.off_ctrl);
     EmitParams ep{};
@@ -395,11 +421,15 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     bp.ngrp = (want & NN_WANT_NODES) ? (uint64_t)p.B * p.groups : 0;
 
     mark(1);
-    if (launch_hist(ep, p.emit_smem, s) != cudaSuccess) return NN_ERR_CUDA;
+    if (!p.direct && launch_hist(ep, p.emit_smem, s) != cudaSuccess) return NN_ERR_CUDA;
     mark(2);
-    if (launch_offsets(op, s) != cudaSuccess) return NN_ERR_CUDA;
+    if (!p.direct && launch_offsets(op, s) != cudaSuccess) return NN_ERR_CUDA;
     mark(3);
-    if (p.fmt.cshift >= 0) {
+    if (p.direct) {
+        bp.direct = DirectMesh{p.type, p.N, p.T, m->n_conn, m->conn, m->elem_ptr, m->elem_type,
+                               (uint32_t)p.bucket_smem, (uint32_t)p.queue_cap};
+        mark(4);
+    } else if (p.fmt.cshift >= 0) {
         if (launch_part_coarse(ep, s) != cudaSuccess) return NN_ERR_CUDA;
         mark(4);
         if (launch_part_fine(ep, op.bstart, p.G_fine, s) != cudaSuccess) return NN_ERR_CUDA;
@@ -408,7 +438,8 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
         mark(4);
     }
     mark(5);
-    if (launch_bucket(bp, p.bucket_grid, p.bucket_threads, p.bucket_smem, s) != cudaSuccess)
+    if (p.direct ? launch_bucket(bp, (int)p.B, p.bucket_threads, p.bucket_smem + (size_t)p.queue_cap * 4, s) != cudaSuccess
+                 : launch_bucket(bp, p.bucket_grid, p.bucket_threads, p.bucket_smem, s) != cudaSuccess)
         return NN_ERR_CUDA;
     mark(6);
     if (want & NN_WANT_NODES) {
@@ -695,7 +726,7 @@ nn_status nn_create(nn_handle** out) {
     h->smem_per_sm = (size_t)per_sm;
     h->bucket_smem = h->smem_optin - 1024;  // the bucket kernel has a little static shared memory
     if (const char* e = std::getenv("NN_SB")) h->sb_override = std::atoi(e);
-    if (const char* e = std::getenv("NN_PART")) h->part_mode = std::strcmp(e, "scatter") == 0 ? 0 : -1;
+    if (const char* e = std::getenv("NN_PART")) h->part_mode = std::strcmp(e, "scatter") == 0 ? 0 : (std::strcmp(e, "sorted") == 0 ? 1 : -1);
     if (const char* e = std::getenv("NN_HIST_CHUNK")) h->hist_chunk_override = std::atoll(e);
     if (const char* e = std::getenv("NN_EMIT_CTAS")) h->emit_ctas_override = std::atoi(e);
     if (const char* e = std::getenv("NN_BUCKET_SMEM_KB")) {
@@ -769,9 +800,12 @@ nn_status nn_plan_info(nn_handle* h, const nn_mesh* mesh, int want, int64_t* inf
     Plan p;
     nn_status st = make_plan(h, mesh, want, &p);
     if (st != NN_OK) return st;
-    const int64_t v[9] = {p.fmt.sb, p.B, p.G, p.fmt.rb, (int64_t)p.ws_min, p.bucket_grid, p.bucket_threads,
-                          (int64_t)p.bucket_smem, p.fmt.cshift};
-    for (int i = 0; i < n && i < 9; ++i) info[i] = v[i];
+    // initialization, histogram, offsets and partition unless direct, buckets, placement of node rows
+    const int64_t kernels = 2 + (p.direct ? 0 : 3 + (p.fmt.cshift > 0)) +
+                            (want & NN_WANT_NODES ? (p.B * p.groups <= NODE_SUM_GROUPS ? 1 : 2) : 0);
+    const int64_t v[10] = {p.fmt.sb, p.B, p.G, p.fmt.rb, (int64_t)p.ws_min, p.bucket_grid, p.bucket_threads,
+                           (int64_t)p.bucket_smem, p.fmt.cshift, p.N > 0 ? kernels : 0};
+    for (int i = 0; i < n && i < 10; ++i) info[i] = v[i];
     return NN_OK;
 }
 

@@ -6,8 +6,10 @@ namespace nn {
 
 cudaError_t launch_bucket_16(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_bucket_32(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
+cudaError_t launch_bucket_direct(const BucketParams& p, int grid, size_t smem, cudaStream_t s);
 cudaError_t set_bucket_smem_16(size_t bytes);
 cudaError_t set_bucket_smem_32(size_t bytes);
+cudaError_t set_bucket_smem_direct(size_t bytes);
 cudaError_t bucket_occupancy_16(int* blocks, int threads, size_t smem);
 cudaError_t bucket_occupancy_32(int* blocks, int threads, size_t smem);
 
@@ -18,6 +20,7 @@ size_t bucket_smem_bytes(int sb, int want, int k, int slots, int rb, int list_ca
 
 cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s) {
     if (grid <= 0) return cudaSuccess;
+    if (p.direct.conn) return launch_bucket_direct(p, grid, smem, s);
     if (p.imax == 8) return launch_bucket_t<8>(p, grid, threads, smem, s);
     if (p.imax == 16) return launch_bucket_16(p, grid, threads, smem, s);
     return launch_bucket_32(p, grid, threads, smem, s);
@@ -27,6 +30,7 @@ cudaError_t set_bucket_smem_all(size_t bytes) {
     cudaError_t e = set_bucket_smem_t<8>(bytes);
     if (e == cudaSuccess) e = set_bucket_smem_16(bytes);
     if (e == cudaSuccess) e = set_bucket_smem_32(bytes);
+    if (e == cudaSuccess) e = set_bucket_smem_direct(bytes);
     return e;
 }
 

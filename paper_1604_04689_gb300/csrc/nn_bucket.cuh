@@ -131,9 +131,24 @@ __device__ inline void warp_bitonic_sort(uint32_t* a, uint32_t n) {
     }
 }
 
+// A record of the bucket being built by its whole CTA.  In a direct build the
+// CTA has written it itself (no read-only load).
+template <int RB, bool DIRECT>
+__device__ __forceinline__ Rec own_rec(const uint8_t* base, uint64_t pos) {
+    if constexpr (!DIRECT) {
+        return load_rec<RB>(base, pos);
+    } else if constexpr (RB == 8) {
+        const uint2 v = __ldcg(reinterpret_cast<const uint2*>(base) + pos);
+        return Rec{v.x, v.y, 0u, 0u};
+    } else {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(base) + pos);
+        return Rec{v.x, v.y, v.z, v.w};
+    }
+}
+
 // The element ids of a node's c records (a repeated node's record adds
 // none), collected by its whole warp into row[0..ec) and sorted there.
-template <int RB, int K>
+template <int RB, int K, bool DIRECT>
 __device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, const uint32_t* grp, uint32_t c,
                                            uint32_t* row, uint32_t ec) {
     const uint32_t lane = threadIdx.x & 31;
@@ -143,7 +158,7 @@ __device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, c
         bool keep = false;
         uint32_t e = 0;
         if (s < c) {
-            const Rec x = load_rec<RB>(rp, grp[s]);
+            const Rec x = own_rec<RB, DIRECT>(rp, grp[s]);
             keep = !((rec_side<RB, K>(f, x) >> f.off_nf) & 1u);
             e = rec_elem<RB>(f, x);
         }
@@ -157,13 +172,13 @@ __device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, c
 
 // The distinct neighbours of a node's c records, collected by its whole warp
 // into a[0 .. K c): sorted, the first of every run kept.  Returns their count.
-template <int RB, int K>
+template <int RB, int K, bool DIRECT>
 __device__ __noinline__ uint32_t warp_node_row(const RecFmt& f, const uint8_t* rp, const uint32_t* grp, uint32_t c,
                                                uint32_t* a) {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t nc = (uint64_t)K * c;
     for (uint32_t s = lane; s < c; s += 32) {
-        const Rec x = load_rec<RB>(rp, grp[s]);
+        const Rec x = own_rec<RB, DIRECT>(rp, grp[s]);
 #pragma unroll
         for (int j = 0; j < K; ++j) a[(uint64_t)s * K + j] = rec_nbr<RB>(f, x, j);
     }
@@ -246,8 +261,128 @@ struct Regs {
     static constexpr int MIN_CTAS = IMAX == 8 ? 4 : (IMAX == 16 ? 3 : 2);
 };
 
-template <int RB, int K, int IMAX>
-__global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketParams p) {
+// Direct builds (small meshes): every CTA reads the whole connectivity and
+// keeps the incidences of its own bucket, so that the histogram, the offsets
+// and the partition are not needed: for a few thousand elements each of those
+// is a launch with next to nothing to do.  What bounds it is the latency of a
+// few dependent steps (triangles 64^2, 128 CTAs: 13 us of a build of 18), so a
+// CTA has as many threads as the registers allow.  Whole builds, graph
+// replays: triangles 64^2 33 -> 18.5 us, hex 21^3 32 -> 27 us; as calls, one
+// after another, triangles 64^2 44 -> 24 us.  scan_elements looks at the elements
+// [e0, e1): incidences of the nodes [v0, v0 + span) go into the queue (element
+// * 8 + local node), and those of lower nodes are counted (below[0]; below[1]:
+// the repeated-node ones), which gives the bucket's place in the results.
+template <int TYPE>
+__device__ __noinline__ void scan_elements(DirectMesh d, uint32_t v0, uint32_t span, uint32_t e0, uint32_t e1,
+                                           uint32_t* queue, uint32_t* n_queue, uint32_t* below, int32_t* status) {
+    constexpr int NPE = TYPE == NN_MIXED ? 8 : ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::NPE;
+    constexpr int U = NPE == 8 ? 2 : 4;  // elements a thread loads at once
+    const uint32_t N = (uint32_t)d.n_nodes, T = blockDim.x;
+    uint32_t less = 0, less_rep = 0;
+    for (uint32_t b = e0 + threadIdx.x; b < e1; b += U * T) {
+        uint32_t nd[U][NPE];
+        uint32_t npe[U];  // 0: no element here
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const uint32_t e = b + q * T;
+            npe[q] = e < e1 ? NPE : 0;
+#pragma unroll
+            for (int i = 0; i < NPE; ++i) nd[q][i] = N;
+            if constexpr (TYPE == NN_TRI) {
+                if (e < e1) {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) nd[q][i] = (uint32_t)__ldg(d.conn + 3 * (size_t)e + i);
+                }
+            } else if constexpr (TYPE == NN_MIXED) {
+                if (e < e1) {
+                    const int t = __ldg(d.elem_type + e);
+                    const int64_t a = __ldg(d.elem_ptr + e), z = __ldg(d.elem_ptr + e + 1);
+                    if (t > NN_HEX || a < 0 || z > d.n_conn || z - a != npe_of(t)) {
+                        set_status(status, NN_ERR_ELEM_PTR);
+                        npe[q] = 0;
+                    } else {
+                        npe[q] = (uint32_t)(z - a);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (i < (int)npe[q]) nd[q][i] = (uint32_t)__ldg(d.conn + a + i);
+                    }
+                }
+            } else {
+                if (e < e1) {
+#pragma unroll
+                    for (int i = 0; i < NPE; i += 4) {
+                        const uint4 x = __ldg(reinterpret_cast<const uint4*>(d.conn + (size_t)NPE * e + i));
+                        nd[q][i] = x.x; nd[q][i + 1] = x.y; nd[q][i + 2] = x.z; nd[q][i + 3] = x.w;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            // (a mixed element's places past its own nodes hold N: neither below v0 nor in the span)
+            uint32_t top = 0;
+            bool rep = false;
+#pragma unroll
+            for (int i = 0; i < NPE; ++i) {
+                top = max(top, TYPE != NN_MIXED || i < (int)npe[q] ? nd[q][i] : 0u);
+#pragma unroll
+                for (int j = 0; j < i; ++j) rep = rep || (nd[q][j] == nd[q][i] && (TYPE != NN_MIXED || i < (int)npe[q]));
+            }
+            if (npe[q] == 0) continue;
+            if (top >= N) {
+                set_status(status, NN_ERR_NODE_RANGE);
+                continue;
+            }
+#pragma unroll
+            for (int i = 0; i < NPE; ++i) {
+                less += nd[q][i] < v0;
+                if (nd[q][i] - v0 < span && nd[q][i] < N) queue[atomicAdd(n_queue, 1u)] = (b + q * T) * 8u + i;
+            }
+            if (rep) {
+#pragma unroll
+                for (int i = 1; i < NPE; ++i) {
+                    bool again = false;
+#pragma unroll
+                    for (int j = 0; j < i; ++j) again = again || nd[q][j] == nd[q][i];
+                    less_rep += again && nd[q][i] < v0;
+                }
+            }
+        }
+    }
+    less = __reduce_add_sync(FULL, less);
+    less_rep = __reduce_add_sync(FULL, less_rep);
+    if ((threadIdx.x & 31) == 0) {
+        if (less) atomicAdd(&below[0], less);
+        if (less_rep) atomicAdd(&below[1], less_rep);
+    }
+}
+
+// The record of local node i of element e (a queue entry of scan_elements).
+template <int RB>
+__device__ __forceinline__ Rec direct_rec(const DirectMesh& d, const RecFmt& f, uint32_t entry) {
+    const uint32_t e = entry >> 3;
+    const int i = (int)(entry & 7u);
+    const int t = d.type == NN_MIXED ? (int)__ldg(d.elem_type + e) : d.type;
+    const int32_t* nd = d.conn + (d.type == NN_MIXED ? __ldg(d.elem_ptr + e) : (int64_t)e * npe_of(t));
+    const int32_t v = __ldg(nd + i);
+    const int K = k_of(t);
+    uint32_t n[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const int32_t y = s < K ? __ldg(nd + nbr_of(t, i, s)) : v;
+        n[s] = y == v ? f.nmask : (uint32_t)y;
+    }
+    uint32_t nf = 0;
+    for (int j = 0; j < i; ++j) nf |= __ldg(nd + j) == v;
+    return pack_rec<RB>(f, make_side(f, (uint32_t)v, nf), e, n, K);
+}
+
+// Threads of a direct build's CTA: as many as the variant's registers allow,
+// for the walk over the connectivity.
+__host__ __device__ constexpr int direct_threads(int imax) { return imax == 8 ? 1024 : 512; }
+
+template <int RB, int K, int IMAX, bool DIRECT>
+__global__ void __launch_bounds__(DIRECT ? direct_threads(IMAX) : 256, DIRECT ? 1 : Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketParams p) {
     constexpr int VE = Regs<K, IMAX>::VE, NW = Regs<K, IMAX>::NW;
     constexpr int U = 4;  // records a thread loads at once
     extern __shared__ __align__(16) uint8_t smem[];
@@ -258,6 +393,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
     __shared__ uint64_t sh_scan[34];
     __shared__ RecFmt sh_fmt;         // for the out-of-line helpers
     __shared__ uint64_t sh_spill[2];  // this CTA's part of the spill area: first word, words
+    __shared__ uint32_t sh_direct[DIRECT ? 6 : 1];  // queue entries, records below (repeated), own (repeated), written
     const bool batched = p.batch.hdr != nullptr;
     const RecFmt f = batched ? p.batch.hdr->fmt : p.fmt;
     const int64_t n_buckets = batched ? p.batch.hdr->n_buckets : p.n_buckets;
@@ -321,17 +457,53 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
     if (tid == 0) {
         sh_spill[0] = sh_spill[1] = 0;
         sh_fmt = f;
-        take(0, atomicAdd(p.ticket, 1u));
+        if constexpr (DIRECT) {
+            meta[0] = BucketMeta{(int64_t)blockIdx.x, 0, 0, 0, 0};
+            for (uint32_t& x : sh_direct) x = 0;
+        } else {
+            take(0, atomicAdd(p.ticket, 1u));
+        }
     }
+    // direct builds: sink(record) for every record of bucket b
+    auto gather = [&](int64_t b, auto&& sink) {
+        uint32_t* const queue = reinterpret_cast<uint32_t*>(smem + p.direct.queue_off);
+        const DirectMesh d = p.direct;
+        const uint32_t v0 = (uint32_t)(b << f.sb), T_e = (uint32_t)d.n_elems;
+        const int npe = d.type == NN_MIXED ? 8 : npe_of(d.type);
+        auto flush = [&]() {
+            const uint32_t n = sh_direct[0];
+            for (uint32_t i = tid; i < n; i += T) sink(direct_rec<RB>(d, f, queue[i]));
+            __syncthreads();
+            if (tid == 0) sh_direct[0] = 0;
+            __syncthreads();
+        };
+        for (uint32_t e = 0; e < T_e;) {
+            // as many elements as the queue surely has room for
+            if ((d.queue_cap - sh_direct[0]) / npe < min(T_e - e, d.queue_cap / npe / 2)) flush();
+            const uint32_t e1 = min(T_e, e + (d.queue_cap - sh_direct[0]) / npe);
+            __syncthreads();
+            int32_t* const st = p.status;
+            switch (d.type) {
+                case NN_TRI: scan_elements<NN_TRI>(d, v0, NB, e, e1, queue, &sh_direct[0], &sh_direct[1], st); break;
+                case NN_QUAD: scan_elements<NN_QUAD>(d, v0, NB, e, e1, queue, &sh_direct[0], &sh_direct[1], st); break;
+                case NN_TET: scan_elements<NN_TET>(d, v0, NB, e, e1, queue, &sh_direct[0], &sh_direct[1], st); break;
+                case NN_HEX: scan_elements<NN_HEX>(d, v0, NB, e, e1, queue, &sh_direct[0], &sh_direct[1], st); break;
+                default: scan_elements<NN_MIXED>(d, v0, NB, e, e1, queue, &sh_direct[0], &sh_direct[1], st); break;
+            }
+            __syncthreads();
+            e = e1;
+        }
+        flush();
+    };
     __syncthreads();
     for (int it = 0;; ++it) {
         const int cur = it & 1;
-        const BucketMeta M = meta[cur];
+        BucketMeta M = meta[cur];
         const int64_t b = M.b;
         if (b >= n_buckets) break;
         uint32_t nx = 0;
         if (tid == 0) {
-            nx = atomicAdd(p.ticket, 1u);  // the next bucket
+            nx = DIRECT ? (uint32_t)n_buckets : atomicAdd(p.ticket, 1u);  // the next bucket
             // the mesh this bucket belongs to (the only one unless batched)
             BucketOut o{p.n_nodes, 0, b == n_buckets - 1, p.rp_n, p.col_n, p.cap_n, p.rp_e, p.col_e, p.cap_e, p.status};
             if (batched) {
@@ -351,11 +523,54 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
         uint32_t* const c32 = cnts + (size_t)cur * 3 * NB;  // [NB] records
         uint32_t* const nfc = c32 + NB;                     // [NB] repeated-node records
         uint32_t* const first = nfc + NB;                   // [NB] first listed record
+        // 1. records into their nodes' columns
+        auto place = [&](const Rec& x) {
+            const uint32_t side = rec_side<RB, K>(f, x), v = side & vmask;
+            const uint32_t s = atomicAdd(&c32[v], 1u);
+            const bool nf = want_e && ((side >> f.off_nf) & 1u);
+            if (nf) atomicAdd(&nfc[v], 1u);
+            if (s < (uint32_t)C) {
+                uint32_t* const col = table + ((v >> 5) * (uint32_t)GW + (v & 31));
+                if (want_e) col[s * 32] = nf ? EMPTY : rec_elem<RB>(f, x);
+                if (want_n) {
+#pragma unroll
+                    for (int j = 0; j < K; ++j)
+                        col[(EC + s * K + j) * 32] = rec_nbr<RB>(f, x, j);
+                }
+            } else {
+                const uint32_t i = atomicAdd(&sh_list[cur], 1u);
+                if (i < (uint32_t)p.list_cap && s < (uint32_t)VE) {
+                    put_rec<RB>(list, i, x);
+                    link[i] = (uint16_t)atomicExch(&first[v], i);
+                } else {
+                    sh_big[cur] = 1;
+                }
+            }
+        };
+        if constexpr (DIRECT) {
+            gather(b, place);
+            for (int l = tid; l < NB; l += T) {
+                if (c32[l]) atomicAdd(&sh_direct[3], c32[l]);
+                if (nfc[l]) atomicAdd(&sh_direct[4], nfc[l]);
+            }
+            __syncthreads();
+            M.r0 = sh_direct[1];
+            M.r1 = M.r0 + sh_direct[3];
+            M.ge = M.r0 - sh_direct[2];
+            M.ne = sh_direct[3] - sh_direct[4];
+            if (M.r1 > p.rec_count) {  // elements of an invalid elem_ptr that overlap: more records than connectivity
+                if (tid == 0) {
+                    set_status(p.status, NN_ERR_WORKSPACE);
+                    sh_big[cur] = 0;
+                }
+                for (int l = tid; l < 2 * NB; l += T) c32[l] = 0;
+                M = BucketMeta{b, 0, 0, 0, 0};
+                __syncthreads();
+            }
+        }
         const uint32_t R = M.r1 - M.r0;
         const uint8_t* const rp = p.rec + (uint64_t)M.r0 * RB;
-
-        // 1. records into their nodes' columns
-        for (uint32_t rb = 0; rb < R; rb += U * T) {
+        for (uint32_t rb = 0; !DIRECT && rb < R; rb += U * T) {
             Rec x[U];
 #pragma unroll
             for (int q = 0; q < U; ++q)
@@ -363,27 +578,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
 #pragma unroll
             for (int q = 0; q < U; ++q) {
                 if (rb + q * T + tid >= R) break;
-                const uint32_t side = rec_side<RB, K>(f, x[q]), v = side & vmask;
-                const uint32_t s = atomicAdd(&c32[v], 1u);
-                const bool nf = want_e && ((side >> f.off_nf) & 1u);
-                if (nf) atomicAdd(&nfc[v], 1u);
-                if (s < (uint32_t)C) {
-                    uint32_t* const col = table + ((v >> 5) * (uint32_t)GW + (v & 31));
-                    if (want_e) col[s * 32] = nf ? EMPTY : rec_elem<RB>(f, x[q]);
-                    if (want_n) {
-#pragma unroll
-                        for (int j = 0; j < K; ++j)
-                            col[(EC + s * K + j) * 32] = rec_nbr<RB>(f, x[q], j);
-                    }
-                } else {
-                    const uint32_t i = atomicAdd(&sh_list[cur], 1u);
-                    if (i < (uint32_t)p.list_cap && s < (uint32_t)VE) {
-                        put_rec<RB>(list, i, x[q]);
-                        link[i] = (uint16_t)atomicExch(&first[v], i);
-                    } else {
-                        sh_big[cur] = 1;
-                    }
-                }
+                place(x[q]);
             }
         }
         __syncthreads();
@@ -558,6 +753,10 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
         if (sh_out.last && tid == 0 && want_e && NN_IN(N, N + 1, status)) sh_out.rp_e[N] = (int64_t)(M.ge + M.ne);
         __syncthreads();
         if (!sh_big[cur]) continue;
+        if constexpr (DIRECT) {  // the records, where a partition would have put them
+            uint8_t* const dst = const_cast<uint8_t*>(rp);
+            gather(b, [&](const Rec& x) { put_rec<RB>(dst, atomicAdd(&sh_direct[5], 1u), x); });
+        }
 
         // 3. the whole CTA: records grouped by node in the spill area, then
         // one warp per group, node by node; rows are sorted in the warp's
@@ -595,7 +794,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
         const bool ok = sh_spill[1] >= need;
         uint32_t* const grp = p.spill + sh_spill[0];
         for (uint32_t r = tid; ok && r < R; r += T)
-            grp[atomicAdd(&cursor[rec_side<RB, K>(f, load_rec<RB>(rp, r)) & vmask], 1u)] = r;
+            grp[atomicAdd(&cursor[rec_side<RB, K>(f, own_rec<RB, DIRECT>(rp, r)) & vmask], 1u)] = r;
         __syncthreads();
         uint32_t* const scratch = table + 2 * NB + warp * scratch_words;
         for (int g = warp; g < GP; g += W) {
@@ -609,7 +808,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
                 if (want_e) {
                     if (lane == 0 && NN_IN(v0 + l, N + 1, status)) sh_out.rp_e[v0 + l] = (int64_t)(M.ge + eoff[l]);
                     if (ok && e_ok && c) {
-                        warp_elem_row<RB, K>(sh_fmt, rp, grp + o, c, a, ec);
+                        warp_elem_row<RB, K, DIRECT>(sh_fmt, rp, grp + o, c, a, ec);
                         for (uint32_t k = lane; k < ec; k += 32) sh_out.col_e[M.ge + eoff[l] + k] = (int32_t)a[k];
                         __syncwarp();
                     }
@@ -617,7 +816,7 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
                 if (want_n) {
                     uint32_t u = 0;
                     if (ok && c) {
-                        u = warp_node_row<RB, K>(sh_fmt, rp, grp + o, c, a);
+                        u = warp_node_row<RB, K, DIRECT>(sh_fmt, rp, grp + o, c, a);
                         const size_t d = (size_t)K * (M.r0 + pr) + run;
                         if (u == 0 || NN_IN(d + u - 1, p.ntmp_words, status))
                             for (uint32_t k = lane; k < u; k += 32) p.ntmp[d + k] = a[k];
@@ -637,41 +836,41 @@ __global__ void __launch_bounds__(256, Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketP
 
 // Allow up to `bytes` of dynamic shared memory, less the kernel's own static
 // shared memory (the sum may not exceed the per-block opt-in limit).
-template <int RB, int K, int IMAX>
+template <int RB, int K, int IMAX, bool DIRECT>
 cudaError_t set_attr(size_t bytes) {
     cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, k_bucket<RB, K, IMAX>);
+    cudaError_t e = cudaFuncGetAttributes(&a, k_bucket<RB, K, IMAX, DIRECT>);
     if (e != cudaSuccess) return e;
     const size_t dyn = bytes > a.sharedSizeBytes ? bytes - a.sharedSizeBytes : 0;
-    return cudaFuncSetAttribute(k_bucket<RB, K, IMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    return cudaFuncSetAttribute(k_bucket<RB, K, IMAX, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
 }
 
 // Launcher, shared-memory limit and occupancy of the IMAX variants (one
 // translation unit each, so that they compile side by side).
-template <int IMAX>
+template <int IMAX, bool DIRECT = false>
 cudaError_t launch_bucket_t(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s) {
     if (p.fmt.rb == 8) {
-        if (p.fmt.k == 2) k_bucket<8, 2, IMAX><<<grid, threads, smem, s>>>(p);
-        else k_bucket<8, 3, IMAX><<<grid, threads, smem, s>>>(p);
+        if (p.fmt.k == 2) k_bucket<8, 2, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
+        else k_bucket<8, 3, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
     } else {
-        if (p.fmt.k == 2) k_bucket<16, 2, IMAX><<<grid, threads, smem, s>>>(p);
-        else k_bucket<16, 3, IMAX><<<grid, threads, smem, s>>>(p);
+        if (p.fmt.k == 2) k_bucket<16, 2, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
+        else k_bucket<16, 3, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
     }
     return cudaGetLastError();
 }
 
-template <int IMAX>
+template <int IMAX, bool DIRECT = false>
 cudaError_t set_bucket_smem_t(size_t bytes) {
-    cudaError_t e = set_attr<8, 2, IMAX>(bytes);
-    if (e == cudaSuccess) e = set_attr<8, 3, IMAX>(bytes);
-    if (e == cudaSuccess) e = set_attr<16, 2, IMAX>(bytes);
-    if (e == cudaSuccess) e = set_attr<16, 3, IMAX>(bytes);
+    cudaError_t e = set_attr<8, 2, IMAX, DIRECT>(bytes);
+    if (e == cudaSuccess) e = set_attr<8, 3, IMAX, DIRECT>(bytes);
+    if (e == cudaSuccess) e = set_attr<16, 2, IMAX, DIRECT>(bytes);
+    if (e == cudaSuccess) e = set_attr<16, 3, IMAX, DIRECT>(bytes);
     return e;
 }
 
 template <int IMAX>
 cudaError_t bucket_occupancy_t(int* blocks, int threads, size_t smem) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_bucket<16, 3, IMAX>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_bucket<16, 3, IMAX, false>, threads, smem);
 }
 
 }  // namespace

@@ -6,6 +6,8 @@
 // (single pass, decoupled lookback over tiles of groups), and a copy of every
 // group's rows to its offset in the mesh's col, with the row pointers.  No
 // bucket ever waits for another while it builds its rows.
+#include <algorithm>
+
 #include "nn_device.cuh"
 
 namespace nn {
@@ -52,7 +54,10 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_node_scan(CompactParams p) {
     }
 }
 
-// One warp per group of 32 nodes.
+// One warp per group of 32 nodes.  SUM: a CTA takes 8 groups and adds up the
+// totals of the groups before them itself, which for a few thousand groups
+// costs less than the scan's launch.
+template <bool SUM>
 __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
     const bool batched = p.batch.hdr != nullptr;
     const int64_t B = batched ? p.batch.hdr->n_buckets : p.n_buckets;
@@ -61,6 +66,16 @@ __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
     const int n_meshes = batched ? p.batch.hdr->n_meshes : 1;
     const int GP = groups_of(sb), lane = threadIdx.x & 31;
     const int64_t n = B * GP, warps = (int64_t)gridDim.x * (COPY_THREADS / 32);
+    uint64_t before = 0;  // SUM: entries of this warp's group's predecessors
+    if constexpr (SUM) {
+        __shared__ uint64_t sh_scan[33];
+        const int64_t first = (int64_t)blockIdx.x * (COPY_THREADS / 32), mine = first + (threadIdx.x >> 5);
+        uint64_t x = 0, total;
+        for (int64_t i = threadIdx.x; i < first; i += COPY_THREADS) x += __ldg(&p.grp[i].y);
+        block_excl_scan(x, &total, sh_scan);
+        before = total;
+        for (int64_t i = first; i < mine && i < n; ++i) before += __ldg(&p.grp[i].y);
+    }
     for (int64_t gi = (int64_t)blockIdx.x * (COPY_THREADS / 32) + (threadIdx.x >> 5); gi < n; gi += warps) {
         const int64_t b = gi / GP;
         int64_t first = 0, N = p.n_nodes;
@@ -87,7 +102,7 @@ __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
         const int64_t v0 = ((b - first) << sb) + (gi - b * GP) * 32, left = N - v0;
         if (left <= 0) continue;
         const int nb = (int)min(left, (int64_t)(sb < 5 ? 1 << sb : 32));
-        const uint64_t gn = p.nstart[gi] - p.nstart[first * GP] + (p.base ? (uint64_t)p.base[1] : 0ull);
+        const uint64_t gn = SUM ? before : p.nstart[gi] - p.nstart[first * GP] + (p.base ? (uint64_t)p.base[1] : 0ull);
         const uint2 g = p.grp[gi];
         const size_t loc = ((size_t)b << sb) + (size_t)(gi - b * GP) * 32 + lane;
         if (lane < nb && NN_IN(loc, p.nloc_words, status)) rp[v0 + lane] = (int64_t)(gn + p.nloc[loc]);
@@ -101,6 +116,15 @@ __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
         if (!NN_IN((size_t)K * g.x + (g.y ? g.y - 1 : 0), p.ntmp_words + (g.y ? 0 : 1), status)) continue;
         for (uint32_t i = lane; i < g.y; i += 32) dst[i] = (int32_t)__ldg(src + i);
     }
+}
+
+// The scans' and tickets' words of a build, and its status: one launch in
+// place of two memsets.
+constexpr int INIT_THREADS = 512;
+__global__ void __launch_bounds__(INIT_THREADS) k_init(uint4* w, int64_t n, int32_t* status) {
+    const int64_t i0 = (int64_t)blockIdx.x * INIT_THREADS + threadIdx.x;
+    if (i0 == 0) *status = 0;
+    for (int64_t i = i0; i < n; i += (int64_t)gridDim.x * INIT_THREADS) w[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Chunked builds run one node range after another into the same CSRs; after
@@ -122,8 +146,20 @@ cudaError_t launch_chunk_advance(int64_t* base, const uint32_t* etot, const uint
 cudaError_t launch_node_compact(const CompactParams& p, int copy_grid, cudaStream_t s) {
     const unsigned tiles = (unsigned)((p.n_groups_cap + NODE_SCAN_TILE - 1) / NODE_SCAN_TILE);
     if (tiles == 0) return cudaSuccess;
+    // (a chunked build needs the scan's grand total, a batch starts over at every mesh)
+    if (p.n_groups_cap <= NODE_SUM_GROUPS && !p.batch.hdr && !p.base) {
+        k_node_copy<true><<<(unsigned)((p.n_groups_cap + COPY_THREADS / 32 - 1) / (COPY_THREADS / 32)), COPY_THREADS, 0, s>>>(p);
+        return cudaGetLastError();
+    }
     k_node_scan<<<tiles, SCAN_THREADS, 0, s>>>(p);
-    k_node_copy<<<copy_grid, COPY_THREADS, 0, s>>>(p);
+    k_node_copy<false><<<copy_grid, COPY_THREADS, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init(void* p, size_t bytes, int32_t* status, int sms, cudaStream_t s) {
+    const int64_t n = (int64_t)(bytes / 16);
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(sms, (n + INIT_THREADS - 1) / INIT_THREADS));
+    k_init<<<(unsigned)blocks, INIT_THREADS, 0, s>>>(static_cast<uint4*>(p), n, status);
     return cudaGetLastError();
 }
 

@@ -128,6 +128,18 @@ struct BatchTables {
     const int64_t* weight_off;  // [n_meshes+1] incidences and elements of the meshes before
 };
 
+// A small mesh built without a partition: the connectivity that every CTA of
+// the bucket pass reads (conn == nullptr: not a direct build).
+struct DirectMesh {
+    int type;
+    int64_t n_nodes, n_elems, n_conn;
+    const int32_t* conn;
+    const int64_t* elem_ptr;
+    const uint8_t* elem_type;
+    uint32_t queue_off;  // dynamic shared memory before the queue of incidences
+    uint32_t queue_cap;  // its entries
+};
+
 // Bucket pass: one CTA per bucket (persistent, buckets taken in order),
 // builds the rows of the bucket's 2^sb nodes in groups of 32 (or of 2^sb,
 // if fewer).
@@ -159,6 +171,7 @@ struct BucketParams {
     uint64_t ntmp_words;    // words of ntmp
     uint64_t nloc_words;    // words of nloc
     uint64_t ngrp;          // entries of grp
+    DirectMesh direct;      // single mesh, one bucket per CTA
 };
 
 constexpr int EMIT_THREADS = 1024;
@@ -167,6 +180,10 @@ constexpr int SORT_THREADS = 256;   // tile-sorted partition passes
 constexpr int OFFSETS_THREADS = 128;  // buckets per tile of the offsets scan
 constexpr int OFFSETS_SLICES = 8;     // slices of its histogram rows summed side by side
 constexpr int NODE_SCAN_TILE = 512;  // groups of 32 nodes per tile of the node-row placement's scan
+
+// groups up to which the placement adds up a group's predecessors itself (16
+// loads a thread) instead of launching a scan
+constexpr int64_t NODE_SUM_GROUPS = 4096;
 
 // Placement of the node rows the bucket pass left in scratch (nn_compact.cu).
 struct CompactParams {
@@ -211,6 +228,8 @@ struct AdjParams {
 cudaError_t launch_adjacency(const AdjParams& p, int grid, int sms, cudaStream_t s);
 int adjacency_slots(int type);
 size_t adjacency_scan_tiles(int64_t n_elems);
+// zeroes [p, p + bytes) (both multiples of 16) and the status word
+cudaError_t launch_init(void* p, size_t bytes, int32_t* status, int sms, cudaStream_t s);
 cudaError_t launch_node_compact(const CompactParams& p, int copy_grid, cudaStream_t s);
 // chunked builds: base[0] += *etot, base[1] += *ntot (either may be nullptr)
 cudaError_t launch_chunk_advance(int64_t* base, const uint32_t* etot, const uint64_t* ntot, cudaStream_t s);

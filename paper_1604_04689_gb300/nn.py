@@ -177,7 +177,7 @@ def nn_query(h: int, mesh: NNMesh, want: int):
 
 
 PLAN_KEYS = ("sb", "n_buckets", "emit_ctas", "record_bytes", "ws_min", "bucket_ctas", "bucket_threads",
-             "bucket_smem", "partition")
+             "bucket_smem", "partition", "kernels")
 
 
 def nn_set_tuning(h: int, tuning: Optional[dict]) -> None:
@@ -193,8 +193,8 @@ def nn_set_tuning(h: int, tuning: Optional[dict]) -> None:
 
 
 def nn_plan_info(h: int, mesh: NNMesh, want: int) -> dict:
-    info = (C.c_int64 * 9)()
-    st = lib().nn_plan_info(h, C.byref(mesh), want, info, 9)
+    info = (C.c_int64 * len(PLAN_KEYS))()
+    st = lib().nn_plan_info(h, C.byref(mesh), want, info, len(PLAN_KEYS))
     if st:
         raise NNError(st, "nn_plan_info")
     return dict(zip(PLAN_KEYS, list(info)))

@@ -17,6 +17,7 @@ import pytest
 import oracle
 from paper_1604_04689_gb300 import meshgen as mg
 from paper_1604_04689_gb300 import nn
+from tests.gpu_util import env
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +99,10 @@ def test_checked_build_matches_oracle_with_canaries_intact(lib, name):
         assert (tail == CANARY).all(), "workspace canary overwritten"
     finally:
         lib.nn_destroy(h)
+
+
+@pytest.mark.parametrize("name", list(MESHES))
+def test_checked_partitioned_build_with_canaries_intact(lib, name):
+    # meshes this small are built without a partition unless told otherwise
+    with env(NN_PART="sorted"):
+        test_checked_build_matches_oracle_with_canaries_intact(lib, name)
