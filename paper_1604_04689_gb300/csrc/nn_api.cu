@@ -210,8 +210,8 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     p.G = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sms * cps, (n_units + 2047) / 2048));
     if (h->emit_ctas_override > 0) p.G = std::min(p.G, h->emit_ctas_override);
     p.G_part = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sms * 2, (n_units + 511) / 512));
-    if (f.cshift >= 0)  // tile-sorted passes: 256-thread CTAs, several per SM
-        p.G_part = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sms * 4, (n_units + 511) / 512));
+    if (f.cshift >= 0)  // tile-sorted passes: 256-thread CTAs, as many as are resident
+        p.G_part = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sms * coarse_ctas_per_sm(p.type), (n_units + 511) / 512));
     p.G_fine = h->sms;  // the fine pass sizes its grid by its occupancy
 
     p.bucket_smem = bucket_smem_bytes(sb, want, p.k, p.slots, f.rb, p.list_cap);

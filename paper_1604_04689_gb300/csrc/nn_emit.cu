@@ -56,6 +56,18 @@ __device__ __forceinline__ void load_mixed_nodes(const int32_t* conn, int64_t a,
     }
 }
 
+// Type and connectivity range of a mixed mesh's element.
+struct MixedHead {
+    int t;
+    int64_t a, b;
+    __device__ __forceinline__ bool valid(const EmitParams& p) const {
+        return t <= NN_HEX && a >= 0 && b <= p.n_conn && b - a == npe_of(t);
+    }
+};
+__device__ __forceinline__ MixedHead load_head(const EmitParams& p, int64_t e) {
+    return MixedHead{__ldg(p.elem_type + e), __ldg(p.elem_ptr + e), __ldg(p.elem_ptr + e + 1)};
+}
+
 // Per-incidence callback signature: (v, nf, e, x0, x1, x2) with x_s = -1 for none.
 template <int TYPE, class F>
 __device__ __forceinline__ void visit_elem(const int32_t* nd, int64_t e, int64_t n_nodes, int32_t* status,
@@ -66,7 +78,7 @@ __device__ __forceinline__ void visit_elem(const int32_t* nd, int64_t e, int64_t
     bool ok = true;
 #pragma unroll
     for (int i = 0; i < NPE; ++i)
-        if (i < npe && (nd[i] < 0 || (int64_t)nd[i] >= n_nodes)) ok = false;
+        if (i < npe && (uint32_t)nd[i] >= (uint32_t)n_nodes) ok = false;  // (n_nodes is below 2^31)
     if (!ok) {
         set_status(status, NN_ERR_NODE_RANGE);
         return;
@@ -99,6 +111,8 @@ __device__ __forceinline__ void walk_cta(const EmitParams& p, F&& f) {
     constexpr int UNIT = TYPE == NN_TRI ? 4 : 1;
     const int64_t n_units = (p.n_elems + UNIT - 1) / UNIT;
     const int64_t u0 = n_units * blockIdx.x / gridDim.x, u1 = n_units * (blockIdx.x + 1) / gridDim.x;
+    MixedHead head{};
+    if (TYPE == NN_MIXED && u0 + threadIdx.x < u1) head = load_head(p, u0 + threadIdx.x);
     for (int64_t u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
         if constexpr (TYPE == NN_TRI) {
             const int64_t e0 = u * 4;
@@ -124,16 +138,16 @@ __device__ __forceinline__ void walk_cta(const EmitParams& p, F&& f) {
             int4 a = __ldg(c4), b = __ldg(c4 + 1);
             int32_t nd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
             visit_elem<NN_HEX>(nd, u, p.n_nodes, p.status, NN_HEX, f);
-        } else {  // mixed
-            const int t = __ldg(p.elem_type + u);
-            const int64_t a = __ldg(p.elem_ptr + u), b = __ldg(p.elem_ptr + u + 1);
-            if (t > NN_HEX || a < 0 || b > p.n_conn || b - a != npe_of(t)) {
+        } else {  // mixed; the next element's type and range are on their way while this one's nodes are read
+            const MixedHead h = head;
+            if (u + blockDim.x < u1) head = load_head(p, u + blockDim.x);
+            if (!h.valid(p)) {
                 set_status(p.status, NN_ERR_ELEM_PTR);
                 continue;
             }
             int32_t nd[8];
-            load_mixed_nodes(p.conn, a, (int)(b - a), nd);
-            visit_elem<NN_MIXED>(nd, u, p.n_nodes, p.status, t, f);
+            load_mixed_nodes(p.conn, h.a, (int)(h.b - h.a), nd);
+            visit_elem<NN_MIXED>(nd, u, p.n_nodes, p.status, h.t, f);
         }
     }
 }
@@ -147,8 +161,14 @@ __device__ __forceinline__ void walk_cta(const EmitParams& p, F&& f) {
 // counters per word.  A count that would pass 65535 carries into its
 // neighbour; the thread whose add would do so sees the old value, flags the
 // CTA, and the CTA counts its slice again with 32-bit counters.
+//
+// What bounds it: ALU instructions (70 to 76 % of that pipe), so ids are
+// checked with one unsigned compare each; in mixed meshes the chain from an
+// element's range to its nodes, so the next element's range is read ahead.
+// GB300, before and now: hex 257^3 158 -> 140 us, tet 161^3 114 -> 99 us,
+// mixed 257^3 531 -> 395 us.
 template <int TYPE, bool RANGED>
-__global__ void __launch_bounds__(EMIT_THREADS) k_hist(EmitParams p) {
+__global__ void __launch_bounds__(EMIT_THREADS, 2) k_hist(EmitParams p) {
     extern __shared__ uint32_t sh_hist[];  // (no static shared memory: the dynamic part may take the whole limit)
     const int64_t B = p.n_buckets;
     const int sb = p.fmt.sb;
@@ -210,11 +230,10 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_slab_count(EmitParams p, int s
         if (sh_cnt[i]) atomicAdd(&counts[i], sh_cnt[i]);
 }
 
-// Load one work unit (4 triangles or one element); returns the runtime type
-// (the element's own type for mixed meshes) and sets ok[w] for each valid
-// element of the unit.  Invalid elements raise the status and are skipped.
+// The nodes of one work unit (4 triangles, or one element that is not of a
+// mixed mesh), as they are.
 template <int TYPE>
-__device__ __forceinline__ int load_unit(const EmitParams& p, int64_t u, int32_t* nd, bool* ok) {
+__device__ __forceinline__ void load_nodes(const EmitParams& p, int64_t u, int32_t* nd) {
     if constexpr (TYPE == NN_TRI) {
         const int64_t e0 = u * 4;
         if (e0 + 4 <= p.n_elems) {
@@ -227,33 +246,7 @@ __device__ __forceinline__ int load_unit(const EmitParams& p, int64_t u, int32_t
 #pragma unroll
             for (int q = 0; q < 12; ++q) nd[q] = (e0 * 3 + q < p.n_conn) ? __ldg(p.conn + e0 * 3 + q) : 0;
         }
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            bool v = e0 + w < p.n_elems;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) v = v && nd[3 * w + i] >= 0 && (int64_t)nd[3 * w + i] < p.n_nodes;
-            if (!v && e0 + w < p.n_elems) set_status(p.status, NN_ERR_NODE_RANGE);
-            ok[w] = v;
-        }
-        return NN_TRI;
-    } else if constexpr (TYPE == NN_MIXED) {
-        const int t = __ldg(p.elem_type + u);
-        const int64_t a = __ldg(p.elem_ptr + u), b = __ldg(p.elem_ptr + u + 1);
-        if (t > NN_HEX || a < 0 || b > p.n_conn || b - a != npe_of(t)) {
-            set_status(p.status, NN_ERR_ELEM_PTR);
-            ok[0] = false;
-            return NN_HEX;
-        }
-        const int npe = (int)(b - a);
-        load_mixed_nodes(p.conn, a, npe, nd);
-        bool v = true;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (q < npe) v = v && nd[q] >= 0 && (int64_t)nd[q] < p.n_nodes;
-        if (!v) set_status(p.status, NN_ERR_NODE_RANGE);
-        ok[0] = v;
-        return t;
-    } else {
+    } else if constexpr (TYPE != NN_MIXED) {
         constexpr int NPE = ElemT<TYPE>::NPE;
         const int4* c4 = reinterpret_cast<const int4*>(p.conn) + (NPE / 4) * u;
         int4 a = __ldg(c4);
@@ -262,11 +255,46 @@ __device__ __forceinline__ int load_unit(const EmitParams& p, int64_t u, int32_t
             int4 b = __ldg(c4 + 1);
             nd[4] = b.x; nd[5] = b.y; nd[6] = b.z; nd[7] = b.w;
         }
-        bool v = true;
+    }
+}
+
+// Which elements of a loaded unit are valid (mixed: of an element whose range
+// is).  Invalid ones raise the status and are skipped.
+template <int TYPE>
+__device__ __forceinline__ void check_unit(const EmitParams& p, int64_t u, const int32_t* nd, int npe, bool* ok) {
+    constexpr int UNIT = TYPE == NN_TRI ? 4 : 1;
+    constexpr int NPE = TYPE == NN_MIXED ? 8 : ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::NPE;
+    const uint32_t N = (uint32_t)p.n_nodes;  // below 2^31
 #pragma unroll
-        for (int i = 0; i < NPE; ++i) v = v && nd[i] >= 0 && (int64_t)nd[i] < p.n_nodes;
-        if (!v) set_status(p.status, NN_ERR_NODE_RANGE);
-        ok[0] = v;
+    for (int w = 0; w < UNIT; ++w) {
+        const bool in = u * UNIT + w < p.n_elems;
+        bool v = in;
+#pragma unroll
+        for (int i = 0; i < NPE; ++i)
+            if (TYPE != NN_MIXED || i < npe) v = v && (uint32_t)nd[NPE * w + i] < N;
+        if (!v && in) set_status(p.status, NN_ERR_NODE_RANGE);
+        ok[w] = v;
+    }
+}
+
+// Load and check one work unit; returns the runtime type (the element's own
+// type for mixed meshes).
+template <int TYPE>
+__device__ __forceinline__ int load_unit(const EmitParams& p, int64_t u, int32_t* nd, bool* ok) {
+    if constexpr (TYPE == NN_MIXED) {
+        const MixedHead h = load_head(p, u);
+        if (!h.valid(p)) {
+            set_status(p.status, NN_ERR_ELEM_PTR);
+            ok[0] = false;
+            return NN_HEX;
+        }
+        const int npe = (int)(h.b - h.a);
+        load_mixed_nodes(p.conn, h.a, npe, nd);
+        check_unit<TYPE>(p, u, nd, npe, ok);
+        return h.t;
+    } else {
+        load_nodes<TYPE>(p, u, nd);
+        check_unit<TYPE>(p, u, nd, 0, ok);
         return TYPE;
     }
 }
@@ -356,25 +384,15 @@ __global__ void __launch_bounds__(PART_THREADS, 2) k_part(EmitParams p) {
 // contiguously, so global stores are coalesced runs instead of one scattered
 // 16-byte store per record.
 
-// Exclusive scan of hist[0..n) (n <= blockDim.x) into dof; returns the total.
-// Ends with a barrier: every thread may read any dof entry afterwards.
-__device__ __forceinline__ uint32_t tile_scan(const uint32_t* hist, uint32_t* dof, int n, uint64_t* sh) {
-    const uint64_t x = threadIdx.x < n ? hist[threadIdx.x] : 0;
-    uint64_t total;
-    const uint64_t ex = block_excl_scan(x, &total, sh);
-    if (threadIdx.x < n) dof[threadIdx.x] = (uint32_t)ex;
-    __syncthreads();
-    return (uint32_t)total;
-}
-
 template <int TYPE>
 struct SortShape {
     static constexpr int UNIT = TYPE == NN_TRI ? 4 : 1;
     static constexpr int NPE = TYPE == NN_MIXED ? 8 : ElemT<(TYPE == NN_MIXED ? NN_HEX : TYPE)>::NPE;
-    static constexpr int UPT = (TYPE == NN_TET || TYPE == NN_QUAD) ? 2 : 1;
+    static constexpr int UPT = TYPE == NN_TET ? 4 : (TYPE == NN_QUAD ? 2 : 1);  // units per thread
     static constexpr int NI = NPE * UNIT;
     static constexpr int RPT = NI * UPT;
     static constexpr int TILE = SORT_THREADS * RPT;
+    static constexpr int CTAS = UPT == 4 ? 3 : 4;  // per SM
 };
 
 template <int TYPE>
@@ -401,16 +419,29 @@ constexpr size_t FINE_SMEM = fine_smem(FINE_DIGITS, 16);
 
 // First (or only) pass: records from the connectivity, radix digit = coarse
 // region (two levels) or bucket (one level, at most 256 buckets).
+//
+// What bounds it: how long the runs are that a tile writes to each region (the
+// lines are filled by parts), then shared-memory traffic (each record is
+// counted, placed and read back).  The next tile's nodes are on their way
+// while this one is written (a mixed mesh: its types and ranges while this one
+// is counted), the cursors' atomics while its records are placed, and a tile
+// has four barriers instead of eight.  Tets: tiles of 4096 records and 3 CTAs
+// per SM; with 255 regions, tiles of 1024 records took 1058 us for tet 161^3,
+// of 2048 616 us and of 4096 474 us.  For the other types larger tiles were no
+// faster (hex 257^3 575 and 591 us) or left too few CTAs (triangles).
+// GB300, before and now: tet 161^3 566 -> 474 us (4.2 TB/s read and written),
+// its 101^3 element rows 147 -> 86 us, hex 257^3 678 -> 575 us (4.7 TB/s),
+// mixed 257^3 1846 -> 1567 us, triangles 2048^2 with holes 125 -> 113 us.
 template <int TYPE, int RB, bool RANGED>
-__global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
+__global__ void __launch_bounds__(SORT_THREADS, SortShape<TYPE>::CTAS) k_part_coarse(EmitParams p) {
     using S = SortShape<TYPE>;
     constexpr int UNIT = S::UNIT, NPE = S::NPE, UPT = S::UPT, NI = S::NI, TILE = S::TILE;
     extern __shared__ __align__(16) uint8_t sm[];
     uint8_t* odig = sm + (size_t)TILE * RB;
     uint32_t* hist = reinterpret_cast<uint32_t*>(odig + TILE);
     uint32_t* dof = hist + 256;
-    uint32_t* gbase = dof + 256;
-    __shared__ uint64_t sh_scan[34];
+    uint32_t* delta = dof + 256;  // global position less place
+    __shared__ uint32_t sh_warp[SORT_THREADS / 32];
     const RecFmt f = p.fmt;
     const bool two = f.cshift > 0;
     const int dshift = f.sb + (two ? f.cshift : 0);
@@ -418,21 +449,58 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
     uint8_t* dst = two ? p.rec_tmp : p.rec;
     const int64_t n_units = (p.n_elems + UNIT - 1) / UNIT;
     const int64_t u0 = n_units * blockIdx.x / gridDim.x, u1 = n_units * (blockIdx.x + 1) / gridDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t nd[UPT][NI];
+    MixedHead head[UPT];
+    auto heads = [&](int64_t tu) {
+        if constexpr (TYPE == NN_MIXED) {
+#pragma unroll
+            for (int k = 0; k < UPT; ++k) {
+                const int64_t u = tu + k * SORT_THREADS + threadIdx.x;
+                head[k] = MixedHead{NN_HEX, 0, 0};
+                if (u < u1) head[k] = load_head(p, u);
+            }
+        }
+    };
+    auto nodes = [&](int64_t tu) {
+#pragma unroll
+        for (int k = 0; k < UPT; ++k) {
+            const int64_t u = tu + k * SORT_THREADS + threadIdx.x;
+            if (u >= u1) continue;
+            if constexpr (TYPE == NN_MIXED) {
+                if (head[k].valid(p)) load_mixed_nodes(p.conn, head[k].a, (int)(head[k].b - head[k].a), nd[k]);
+            } else {
+                load_nodes<TYPE>(p, u, nd[k]);
+            }
+        }
+    };
+    hist[threadIdx.x] = 0;
+    heads(u0);
+    nodes(u0);
+    __syncthreads();
     for (int64_t tu = u0; tu < u1; tu += (int64_t)SORT_THREADS * UPT) {
-        hist[threadIdx.x] = 0;
-        __syncthreads();
-        int32_t nd[UPT][NI];
         bool ok[UPT][UNIT];
         int t[UPT];
         uint16_t rk[UPT][NI];
         uint8_t dg[UPT][NI];
 #pragma unroll
         for (int k = 0; k < UPT; ++k) {
-            const int64_t u = tu + (int64_t)threadIdx.x * UPT + k;
+            const int64_t u = tu + k * SORT_THREADS + threadIdx.x;
 #pragma unroll
             for (int w = 0; w < UNIT; ++w) ok[k][w] = false;
             t[k] = TYPE == NN_MIXED ? NN_HEX : TYPE;
-            if (u < u1) t[k] = load_unit<TYPE>(p, u, nd[k], ok[k]);
+            if (u < u1) {
+                if constexpr (TYPE == NN_MIXED) {
+                    if (head[k].valid(p)) {
+                        t[k] = head[k].t;
+                        check_unit<TYPE>(p, u, nd[k], npe_of(t[k]), ok[k]);
+                    } else {
+                        set_status(p.status, NN_ERR_ELEM_PTR);
+                    }
+                } else {
+                    check_unit<TYPE>(p, u, nd[k], 0, ok[k]);
+                }
+            }
             const int npe = TYPE == NN_MIXED ? npe_of(t[k]) : NPE;
 #pragma unroll
             for (int j = 0; j < NI; ++j) {
@@ -447,12 +515,34 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
                 }
             }
         }
+        const int64_t next = tu + (int64_t)SORT_THREADS * UPT;
+        heads(next);
         __syncthreads();
-        const uint32_t n_tile = tile_scan(hist, dof, 256, sh_scan);
-        if (hist[threadIdx.x]) gbase[threadIdx.x] = atomicAdd(&cursor[threadIdx.x], hist[threadIdx.x]);
+        // a thread per digit: its place in the tile and its global range
+        const uint32_t h = hist[threadIdx.x];
+        uint32_t inc = h;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (lane == 31) sh_warp[warp] = inc;
+        hist[threadIdx.x] = 0;  // for the next tile
+        uint32_t gb = 0;
+        if (h) gb = atomicAdd(&cursor[threadIdx.x], h);  // (needed only after the placement below)
+        __syncthreads();
+        uint32_t at = inc - h, n_tile = 0;
+#pragma unroll
+        for (int w = 0; w < SORT_THREADS / 32; ++w) {
+            const uint32_t x = sh_warp[w];
+            if (w < warp) at += x;
+            n_tile += x;
+        }
+        dof[threadIdx.x] = at;
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < UPT; ++k) {
-            const int64_t u = tu + (int64_t)threadIdx.x * UPT + k;
+            const int64_t u = tu + k * SORT_THREADS + threadIdx.x;
 #pragma unroll
             for (int j = 0; j < NI; ++j) {
                 if (rk[k][j] == 0xFFFF) continue;
@@ -464,13 +554,14 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_coarse(EmitParams p) {
                 odig[q] = dg[k][j];
             }
         }
+        nodes(next);
+        delta[threadIdx.x] = gb - at;
         __syncthreads();
         for (uint32_t q = threadIdx.x; q < n_tile; q += SORT_THREADS) {
-            const uint32_t d = odig[q];
-            const uint64_t pos = (uint64_t)gbase[d] + (q - dof[d]);
+            const uint32_t pos = delta[odig[q]] + q;
             if (pos < p.rec_cap) put_rec<RB>(dst, pos, take_rec<RB>(sm, q));
         }
-        __syncthreads();
+        // (no barrier: what the next tile writes before its second one is not read here)
     }
 }
 
@@ -789,6 +880,8 @@ cudaError_t part_coarse_t(const EmitParams& p, cudaStream_t s) {
     else coarse_r<TYPE, false>(p, s);
     return cudaGetLastError();
 }
+
+int coarse_ctas_per_sm(int type) { return type == NN_TET ? SortShape<NN_TET>::CTAS : SortShape<NN_HEX>::CTAS; }
 
 cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s) {
     switch (p.type) {

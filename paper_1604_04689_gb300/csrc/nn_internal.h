@@ -240,6 +240,7 @@ cudaError_t launch_part(const EmitParams& p, cudaStream_t s);
 cudaError_t launch_part_sorted(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s);
 // the two passes of launch_part_sorted on their own (the fine pass only when cshift > 0)
 cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s);
+int coarse_ctas_per_sm(int type);
 cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s);
 cudaError_t launch_offsets(const OffsetsParams& p, cudaStream_t s);
 cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
