@@ -399,12 +399,17 @@ template <int TYPE>
 __host__ __device__ constexpr size_t coarse_smem(int rb) {
     return (size_t)SortShape<TYPE>::TILE * (rb + 1) + 3 * 256 * 4;
 }
-// Records per thread of a fine-pass tile: 4, or 8 when a coarse region has
-// at least 512 buckets (then a 1024-record tile has about two records per
-// bucket, and its one cursor atomic per bucket present would come close to
-// one per two records; with 256 buckets the larger tile measured slower).
-constexpr int FINE_RPT_WIDE_DIGITS = 512;
-__host__ __device__ constexpr int fine_rpt(int nd) { return nd >= FINE_RPT_WIDE_DIGITS ? 8 : 4; }
+// Tiles of the fine pass: 16 KB of records, 4 to a thread of 256 (8-byte
+// records 8); 2048 records and 512 threads when a coarse region has at least
+// 512 buckets (then a 1024-record tile has two records per bucket, and its one
+// cursor atomic per bucket present comes close to one per two records: L2
+// atomics, about 40 G/s, bind the pass).  hex 257^3 and mixed 257^3: 256
+// threads of 8 records 943 and 1503 us, 512 of 8 857 and 1366 us, 512 of 4 807
+// and 1285 us.
+constexpr int FINE_WIDE_DIGITS = 512;
+__host__ __device__ constexpr int fine_threads(int nd) { return nd >= FINE_WIDE_DIGITS ? 512 : 256; }
+__host__ __device__ constexpr int fine_rpt(int nd, int rb) { return nd < FINE_WIDE_DIGITS && rb == 8 ? 8 : 4; }
+__host__ __device__ constexpr int fine_tile(int nd, int rb) { return fine_threads(nd) * fine_rpt(nd, rb); }
 constexpr int FINE_DIGITS = 4096;  // buckets per coarse region: at most 256 x 4096 buckets in all
 // shared memory of the fine pass for nd digits per coarse region and rb-byte
 // records: two tile stages (bulk-copy targets, 16 bytes of slack for an odd
@@ -412,8 +417,7 @@ constexpr int FINE_DIGITS = 4096;  // buckets per coarse region: at most 256 x 4
 // first work item and record of every coarse region
 __host__ __device__ constexpr size_t fine_stage_bytes(int tile, int rb) { return (size_t)tile * rb + 16; }
 __host__ __device__ constexpr size_t fine_smem(int nd, int rb) {
-    return 2 * fine_stage_bytes(SORT_THREADS * fine_rpt(nd), rb) + (size_t)SORT_THREADS * fine_rpt(nd) * 2 +
-           3 * (size_t)nd * 4 + 2 * 257 * 4;
+    return 2 * fine_stage_bytes(fine_tile(nd, rb), rb) + (size_t)fine_tile(nd, rb) * 2 + 3 * (size_t)nd * 4 + 2 * 257 * 4;
 }
 constexpr size_t FINE_SMEM = fine_smem(FINE_DIGITS, 16);
 
@@ -581,10 +585,11 @@ __global__ void __launch_bounds__(SORT_THREADS, SortShape<TYPE>::CTAS) k_part_co
 // reservations are held in registers: one size for all cost a third of the
 // resident CTAs).  GB300, before and now: tet 161^3 0.71 -> 0.50 ms (6.3 TB/s
 // read and written), triangles 2048^2 0.172 -> 0.127 ms (6.0 TB/s), hex 257^3
-// (512 digits per region) 1.33 -> 0.94 ms (4.6 TB/s).
-template <int RB, int FINE_RPT, int DPT>
-__global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const uint32_t* bstart) {
-    constexpr int FINE_TILE = SORT_THREADS * FINE_RPT;
+// (512 digits per region) 1.33 -> 0.94 ms, and 0.81 ms (5.3 TB/s) with 512
+// threads; tet 101^3 element rows 0.117 -> 0.092 -> 0.085 ms.
+template <int RB, int THREADS, int FINE_RPT, int DPT>
+__global__ void __launch_bounds__(THREADS) k_part_fine(EmitParams p, const uint32_t* bstart) {
+    constexpr int FINE_TILE = THREADS * FINE_RPT;
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr uint32_t SB = (uint32_t)fine_stage_bytes(FINE_TILE, RB);
     uint8_t* const stage = sm;  // [2][SB]
@@ -598,7 +603,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
     uint32_t* const tpre = delta + nd_;   // [257] first tile of each coarse region
     uint32_t* const rbeg = tpre + 257;    // [257] first record of each coarse region
     __shared__ uint64_t sh_scan[34];
-    __shared__ uint32_t sh_warp[SORT_THREADS / 32];
+    __shared__ uint32_t sh_warp[THREADS / 32];
     __shared__ uint64_t mbar[2];
     __shared__ uint32_t sh_tile[2][4];  // per stage: region, first record, end, offset of record 0 in the stage
     __shared__ int32_t sh_lost;
@@ -625,7 +630,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         mbar_init(&mbar[1]);
         sh_lost = 0;
     }
-    for (int i = tid; i < nd_; i += SORT_THREADS) hist[i] = 0;
+    for (int i = tid; i < nd_; i += THREADS) hist[i] = 0;
     __syncthreads();
     const uint32_t W = tpre[R1];
     // One thread: locate work item wi and start the copy of its records
@@ -653,7 +658,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         }
     };
     if (tid == 0 && blockIdx.x < W) issue(0, blockIdx.x);
-    const int per = nd_ > SORT_THREADS ? nd_ / SORT_THREADS : 1;  // digits of a thread (both are powers of two)
+    const int per = nd_ > THREADS ? nd_ / THREADS : 1;  // digits of a thread (both are powers of two)
     uint32_t par[2] = {0u, 0u};  // parity of each stage's next copy
     int it = 0;
     for (uint32_t wi = blockIdx.x; wi < W; wi += gridDim.x, ++it) {
@@ -678,13 +683,13 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         uint32_t dr[FINE_RPT];
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k) {
-            const uint32_t r = tid + k * SORT_THREADS;
+            const uint32_t r = tid + k * THREADS;
             dr[k] = 0;
             if (r < n) dr[k] = (rec_side<RB, 0>(f, take_rec<RB>(src, r)) >> f.sb) & (uint32_t)(nd_ - 1);
         }
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k)
-            if (tid + k * SORT_THREADS < n) dr[k] |= atomicAdd(&hist[dr[k]], 1u) << 16;
+            if (tid + k * THREADS < n) dr[k] |= atomicAdd(&hist[dr[k]], 1u) << 16;
         __syncthreads();
         // places of the digits, and the reserved global range of each present
         // one (its atomic's answer is needed only after the placement below)
@@ -722,7 +727,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k) {
-            const uint32_t r = tid + k * SORT_THREADS;
+            const uint32_t r = tid + k * THREADS;
             if (r < n) perm[dof[dr[k] & 0xffffu] + (dr[k] >> 16)] = (uint16_t)r;
         }
 #pragma unroll
@@ -731,7 +736,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_part_fine(EmitParams p, const 
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < FINE_RPT; ++k) {
-            const uint32_t q = tid + k * SORT_THREADS;
+            const uint32_t q = tid + k * THREADS;
             if (q < n) {
                 const Rec x = take_rec<RB>(src, perm[q]);
                 const uint32_t pos = delta[(rec_side<RB, 0>(f, x) >> f.sb) & (uint32_t)(nd_ - 1)] + q;
@@ -895,22 +900,23 @@ cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s) {
 
 // One CTA per resident slot (the SMs times the CTAs its shared memory
 // allows per SM): each CTA works through its tiles with the copies in flight.
-template <int RB, int RPT, int DPT>
+template <int RB, int THREADS, int RPT, int DPT>
 cudaError_t fine_t(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
     const size_t fs = fine_smem(1 << p.fmt.cshift, RB);
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_part_fine<RB, RPT, DPT>, SORT_THREADS, fs);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_part_fine<RB, THREADS, RPT, DPT>, THREADS, fs);
     if (e != cudaSuccess) return e;
-    k_part_fine<RB, RPT, DPT><<<std::max(1, sms * std::max(occ, 1)), SORT_THREADS, fs, s>>>(p, bstart);
+    k_part_fine<RB, THREADS, RPT, DPT><<<std::max(1, sms * std::max(occ, 1)), THREADS, fs, s>>>(p, bstart);
     return cudaGetLastError();
 }
 
 template <int RB>
 cudaError_t fine_rb(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
+    constexpr int TN = fine_threads(1), TW = fine_threads(FINE_WIDE_DIGITS);
     const int nd = 1 << p.fmt.cshift;
-    if (nd < FINE_RPT_WIDE_DIGITS) return fine_t<RB, 4, FINE_RPT_WIDE_DIGITS / 2 / SORT_THREADS>(p, bstart, sms, s);
-    if (nd == FINE_RPT_WIDE_DIGITS) return fine_t<RB, 8, FINE_RPT_WIDE_DIGITS / SORT_THREADS>(p, bstart, sms, s);
-    return fine_t<RB, 8, FINE_DIGITS / SORT_THREADS>(p, bstart, sms, s);
+    if (nd < FINE_WIDE_DIGITS) return fine_t<RB, TN, fine_rpt(1, RB), FINE_WIDE_DIGITS / 2 / TN>(p, bstart, sms, s);
+    if (nd == FINE_WIDE_DIGITS) return fine_t<RB, TW, fine_rpt(FINE_WIDE_DIGITS, RB), FINE_WIDE_DIGITS / TW>(p, bstart, sms, s);
+    return fine_t<RB, TW, fine_rpt(FINE_WIDE_DIGITS, RB), FINE_DIGITS / TW>(p, bstart, sms, s);
 }
 
 cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
@@ -920,13 +926,14 @@ cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sm
 
 template <int RB>
 cudaError_t set_fine_smem() {
-    cudaError_t e = cudaFuncSetAttribute(k_part_fine<RB, 4, FINE_RPT_WIDE_DIGITS / 2 / SORT_THREADS>,
+    constexpr int TN = fine_threads(1), TW = fine_threads(FINE_WIDE_DIGITS);
+    cudaError_t e = cudaFuncSetAttribute(k_part_fine<RB, TN, fine_rpt(1, RB), FINE_WIDE_DIGITS / 2 / TN>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_part_fine<RB, 8, FINE_RPT_WIDE_DIGITS / SORT_THREADS>,
+        e = cudaFuncSetAttribute(k_part_fine<RB, TW, fine_rpt(FINE_WIDE_DIGITS, RB), FINE_WIDE_DIGITS / TW>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_part_fine<RB, 8, FINE_DIGITS / SORT_THREADS>,
+        e = cudaFuncSetAttribute(k_part_fine<RB, TW, fine_rpt(FINE_WIDE_DIGITS, RB), FINE_DIGITS / TW>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINE_SMEM);
     return e;
 }
