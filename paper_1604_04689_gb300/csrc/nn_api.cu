@@ -368,6 +368,8 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     ep.rec = w + p.off_rec;
     ep.rec_cap = (uint64_t)p.n_conn;
     ep.status = d_status;
+    ep.chain = p.n_conn <= CHAIN_RECORDS;
+    ep.after_kernel = !base;  // (chunks begin with a memset)
     ep.hist_words = (uint64_t)p.G * (uint64_t)p.B;
 
     OffsetsParams op{};
@@ -385,7 +387,10 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     op.rec_cap = (uint64_t)p.n_conn;
     op.status = d_status;
 
+    op.chain = ep.chain;
+
     BucketParams bp{};
+    bp.chain = ep.chain;
     bp.fmt = p.fmt;
     bp.n_nodes = p.N;
     bp.n_buckets = p.B;
@@ -450,6 +455,7 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
         cp.k = p.k;
         cp.n_nodes = p.N;
         cp.base = base;
+        cp.chain = bp.chain;
         cp.grp = bp.grp;
         cp.nloc = bp.nloc;
         cp.ntmp = bp.ntmp;
@@ -608,6 +614,7 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     if (ws_bytes < bp.ws_min) return NN_ERR_WORKSPACE;
     uint8_t* w = static_cast<uint8_t*>(ws);
     if (cudaMemcpyAsync(w, staging, bp.table_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return NN_ERR_CUDA;
+    const bool chain = c->max_conn <= CHAIN_RECORDS;
     BatchTables bt;
     bt.hdr = reinterpret_cast<const BatchHeader*>(w);
     bt.meshes = reinterpret_cast<const BatchMesh*>(w + bp.meshes_off);
@@ -620,10 +627,10 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     uint32_t* ctrl = reinterpret_cast<uint32_t*>(w + bp.off_ctrl);
     uint64_t* lb_off = reinterpret_cast<uint64_t*>(w + bp.off_lb_off);
     uint8_t* rec = w + bp.off_rec;
-    if (launch_batch_emit(bt, bcount, nfc, gcur, rec, lb_off, ctrl, bp.emit_grid, 0, s,
+    if (launch_batch_emit(bt, bcount, nfc, gcur, rec, lb_off, ctrl, bp.emit_grid, 0, chain, s,
                           reinterpret_cast<uint64_t*>(w + bp.off_lb_ns)) != cudaSuccess)
         return NN_ERR_CUDA;
-    if (launch_batch_emit(bt, bcount, nfc, gcur, rec, lb_off, ctrl, bp.emit_grid, 1, s) != cudaSuccess)
+    if (launch_batch_emit(bt, bcount, nfc, gcur, rec, lb_off, ctrl, bp.emit_grid, 1, chain, s) != cudaSuccess)
         return NN_ERR_CUDA;
     OffsetsParams op{};
     op.hist = bcount;
@@ -638,8 +645,9 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     op.rec_cap = (uint64_t)c->max_conn;
     op.status = reinterpret_cast<int32_t*>(ctrl + 8);  // passed on to every mesh by the bucket pass
     op.hdr = bt.hdr;
+    op.chain = chain;
     if (launch_offsets(op, s) != cudaSuccess) return NN_ERR_CUDA;
-    if (launch_batch_emit(bt, bcount, nfc, gcur, rec, lb_off, ctrl, bp.emit_grid, 2, s) != cudaSuccess)
+    if (launch_batch_emit(bt, bcount, nfc, gcur, rec, lb_off, ctrl, bp.emit_grid, 2, chain, s) != cudaSuccess)
         return NN_ERR_CUDA;
     BucketParams kp{};
     kp.n_buckets = 0;
@@ -656,6 +664,7 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     kp.fmt.rb = 16;
     kp.fmt.k = 3;
     kp.imax = 32;
+    kp.chain = chain;
     kp.slots = BATCH_SLOTS;
     kp.list_cap = BATCH_LIST;
     kp.ntmp = reinterpret_cast<uint32_t*>(w + bp.off_ntmp);
@@ -677,6 +686,7 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
         cp.ticket = ctrl + 4;
         cp.status = reinterpret_cast<int32_t*>(ctrl + 8);
         cp.batch = bt;
+        cp.chain = chain;
         cp.ntmp_words = kp.ntmp_words;
         cp.nloc_words = kp.nloc_words;
         if (launch_node_compact(cp, h->sms * 8, s) != cudaSuccess) return NN_ERR_CUDA;

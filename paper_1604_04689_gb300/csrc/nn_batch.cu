@@ -120,6 +120,7 @@ __device__ __forceinline__ bool shared_buckets(const BatchTables& bt, const Slic
 
 __global__ void __launch_bounds__(BATCH_THREADS) k_batch_init(BatchTables bt, uint32_t* bcount, uint32_t* nfc,
                                                               uint64_t* lb_off, uint32_t* ctrl, uint64_t* lb_ns) {
+    chain_begin();
     const int64_t B = bt.hdr->n_buckets;
     const int64_t tiles = (B + OFFSETS_THREADS - 1) / OFFSETS_THREADS;
     const int n = bt.hdr->n_meshes;
@@ -154,6 +155,7 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_batch_init(BatchTables bt, ui
 // 787 -> 465 us.  A slice with more buckets than counters has few records per
 // bucket to add up, and keeps one global atomic per record.
 __global__ void __launch_bounds__(BATCH_THREADS, 3) k_hist_b(BatchTables bt, uint32_t* bcount, uint32_t* nfc) {
+    chain_begin();
     __shared__ uint32_t cnt[BATCH_COUNTERS];
     const int sb = bt.hdr->fmt.sb;
     const Slice s = cta_slice(bt);
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 3) k_hist_b(BatchTables bt, uin
 // a range is reserved in every bucket it touches, and the second walk (its
 // connectivity is in L2 now) takes places from the ranges.
 __global__ void __launch_bounds__(BATCH_THREADS, 3) k_part_b(BatchTables bt, uint32_t* gcur, uint8_t* rec) {
+    chain_begin();
     __shared__ uint32_t place[BATCH_COUNTERS];
     const RecFmt f = bt.hdr->fmt;
     const uint64_t cap = (uint64_t)bt.hdr->n_records;
@@ -246,11 +249,11 @@ __global__ void __launch_bounds__(BATCH_THREADS, 3) k_part_b(BatchTables bt, uin
 }  // namespace
 
 cudaError_t launch_batch_emit(const BatchTables& bt, uint32_t* bcount, uint32_t* nfc, uint32_t* gcur, uint8_t* rec,
-                              uint64_t* lb_off, uint32_t* ctrl, int grid, int stage, cudaStream_t s,
-                              uint64_t* lb_ns) {
-    if (stage == 0) k_batch_init<<<grid, BATCH_THREADS, 0, s>>>(bt, bcount, nfc, lb_off, ctrl, lb_ns);
-    else if (stage == 1) k_hist_b<<<grid, BATCH_THREADS, 0, s>>>(bt, bcount, nfc);
-    else k_part_b<<<grid, BATCH_THREADS, 0, s>>>(bt, gcur, rec);
+                              uint64_t* lb_off, uint32_t* ctrl, int grid, int stage, bool chain,
+                              cudaStream_t s, uint64_t* lb_ns) {
+    if (stage == 1) return launch_chained(chain, k_hist_b, grid, BATCH_THREADS, 0, s, bt, bcount, nfc);
+    if (stage == 2) return launch_chained(chain, k_part_b, grid, BATCH_THREADS, 0, s, bt, gcur, rec);
+    k_batch_init<<<grid, BATCH_THREADS, 0, s>>>(bt, bcount, nfc, lb_off, ctrl, lb_ns);
     return cudaGetLastError();
 }
 

@@ -383,6 +383,7 @@ __host__ __device__ constexpr int direct_threads(int imax) { return imax == 8 ? 
 
 template <int RB, int K, int IMAX, bool DIRECT>
 __global__ void __launch_bounds__(DIRECT ? direct_threads(IMAX) : 256, DIRECT ? 1 : Regs<K, IMAX>::MIN_CTAS) k_bucket(BucketParams p) {
+    chain_begin();
     constexpr int VE = Regs<K, IMAX>::VE, NW = Regs<K, IMAX>::NW;
     constexpr int U = 4;  // records a thread loads at once
     extern __shared__ __align__(16) uint8_t smem[];
@@ -850,13 +851,11 @@ cudaError_t set_attr(size_t bytes) {
 template <int IMAX, bool DIRECT = false>
 cudaError_t launch_bucket_t(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s) {
     if (p.fmt.rb == 8) {
-        if (p.fmt.k == 2) k_bucket<8, 2, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
-        else k_bucket<8, 3, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
-    } else {
-        if (p.fmt.k == 2) k_bucket<16, 2, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
-        else k_bucket<16, 3, IMAX, DIRECT><<<grid, threads, smem, s>>>(p);
+        return launch_chained(p.chain, p.fmt.k == 2 ? k_bucket<8, 2, IMAX, DIRECT> : k_bucket<8, 3, IMAX, DIRECT>, grid, threads,
+                              smem, s, p);
     }
-    return cudaGetLastError();
+    return launch_chained(p.chain, p.fmt.k == 2 ? k_bucket<16, 2, IMAX, DIRECT> : k_bucket<16, 3, IMAX, DIRECT>, grid, threads,
+                          smem, s, p);
 }
 
 template <int IMAX, bool DIRECT = false>

@@ -21,6 +21,7 @@ constexpr int COPY_THREADS = 256;
 __device__ __forceinline__ int groups_of(int sb) { return sb < 5 ? 1 : 1 << (sb - 5); }
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_node_scan(CompactParams p) {
+    chain_begin();
     __shared__ uint64_t sh_scan[33];
     __shared__ uint32_t sh_tile;
     __shared__ uint64_t sh_base;
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_node_scan(CompactParams p) {
 // costs less than the scan's launch.
 template <bool SUM>
 __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
+    chain_begin();
     const bool batched = p.batch.hdr != nullptr;
     const int64_t B = batched ? p.batch.hdr->n_buckets : p.n_buckets;
     const int sb = batched ? p.batch.hdr->fmt.sb : p.sb;
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
 // place of two memsets.
 constexpr int INIT_THREADS = 512;
 __global__ void __launch_bounds__(INIT_THREADS) k_init(uint4* w, int64_t n, int32_t* status) {
+    chain_begin();
     const int64_t i0 = (int64_t)blockIdx.x * INIT_THREADS + threadIdx.x;
     if (i0 == 0) *status = 0;
     for (int64_t i = i0; i < n; i += (int64_t)gridDim.x * INIT_THREADS) w[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -148,12 +151,11 @@ cudaError_t launch_node_compact(const CompactParams& p, int copy_grid, cudaStrea
     if (tiles == 0) return cudaSuccess;
     // (a chunked build needs the scan's grand total, a batch starts over at every mesh)
     if (p.n_groups_cap <= NODE_SUM_GROUPS && !p.batch.hdr && !p.base) {
-        k_node_copy<true><<<(unsigned)((p.n_groups_cap + COPY_THREADS / 32 - 1) / (COPY_THREADS / 32)), COPY_THREADS, 0, s>>>(p);
-        return cudaGetLastError();
+        return launch_chained(p.chain, k_node_copy<true>, (unsigned)((p.n_groups_cap + COPY_THREADS / 32 - 1) / (COPY_THREADS / 32)),
+                              COPY_THREADS, 0, s, p);
     }
-    k_node_scan<<<tiles, SCAN_THREADS, 0, s>>>(p);
-    k_node_copy<false><<<copy_grid, COPY_THREADS, 0, s>>>(p);
-    return cudaGetLastError();
+    const cudaError_t e = launch_chained(p.chain, k_node_scan, tiles, SCAN_THREADS, 0, s, p);
+    return e == cudaSuccess ? launch_chained(p.chain, k_node_copy<false>, copy_grid, COPY_THREADS, 0, s, p) : e;
 }
 
 cudaError_t launch_init(void* p, size_t bytes, int32_t* status, int sms, cudaStream_t s) {

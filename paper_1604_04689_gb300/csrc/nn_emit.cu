@@ -169,6 +169,7 @@ __device__ __forceinline__ void walk_cta(const EmitParams& p, F&& f) {
 // mixed 257^3 531 -> 395 us.
 template <int TYPE, bool RANGED>
 __global__ void __launch_bounds__(EMIT_THREADS, 2) k_hist(EmitParams p) {
+    chain_begin();
     extern __shared__ uint32_t sh_hist[];  // (no static shared memory: the dynamic part may take the whole limit)
     const int64_t B = p.n_buckets;
     const int sb = p.fmt.sb;
@@ -440,6 +441,7 @@ template <int TYPE, int RB, bool RANGED>
 __global__ void __launch_bounds__(SORT_THREADS, SortShape<TYPE>::CTAS) k_part_coarse(EmitParams p) {
     using S = SortShape<TYPE>;
     constexpr int UNIT = S::UNIT, NPE = S::NPE, UPT = S::UPT, NI = S::NI, TILE = S::TILE;
+    chain_begin();
     extern __shared__ __align__(16) uint8_t sm[];
     uint8_t* odig = sm + (size_t)TILE * RB;
     uint32_t* hist = reinterpret_cast<uint32_t*>(odig + TILE);
@@ -590,6 +592,7 @@ __global__ void __launch_bounds__(SORT_THREADS, SortShape<TYPE>::CTAS) k_part_co
 template <int RB, int THREADS, int FINE_RPT, int DPT>
 __global__ void __launch_bounds__(THREADS) k_part_fine(EmitParams p, const uint32_t* bstart) {
     constexpr int FINE_TILE = THREADS * FINE_RPT;
+    chain_begin();
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr uint32_t SB = (uint32_t)fine_stage_bytes(FINE_TILE, RB);
     uint8_t* const stage = sm;  // [2][SB]
@@ -756,6 +759,7 @@ __global__ void __launch_bounds__(THREADS) k_part_fine(EmitParams p, const uint3
 // for 16,384 and 27 us for 66,308 (23 before).  64 buckets and 16 slices took
 // 17 and 41 us for the last two.
 __global__ void __launch_bounds__(OFFSETS_THREADS * OFFSETS_SLICES) k_offsets(OffsetsParams p) {
+    chain_begin();
     __shared__ uint32_t sh_part[OFFSETS_SLICES][OFFSETS_THREADS];
     __shared__ uint64_t sh_scan[33];
     __shared__ uint32_t sh_tile;
@@ -813,9 +817,8 @@ __global__ void __launch_bounds__(OFFSETS_THREADS * OFFSETS_SLICES) k_offsets(Of
 
 template <int TYPE>
 cudaError_t hist_t(const EmitParams& p, size_t smem, cudaStream_t s) {
-    if (ranged(p)) k_hist<TYPE, true><<<p.n_cta, EMIT_THREADS, smem, s>>>(p);
-    else k_hist<TYPE, false><<<p.n_cta, EMIT_THREADS, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_chained(p.chain && p.after_kernel, ranged(p) ? k_hist<TYPE, true> : k_hist<TYPE, false>, p.n_cta,
+                          EMIT_THREADS, smem, s, p);
 }
 template <int TYPE, bool RANGED>
 void part_r(const EmitParams& p, cudaStream_t s) {
@@ -873,17 +876,14 @@ cudaError_t launch_part(const EmitParams& p, cudaStream_t s) {
 }
 
 template <int TYPE, bool RANGED>
-void coarse_r(const EmitParams& p, cudaStream_t s) {
-    const size_t smem = coarse_smem<TYPE>(p.fmt.rb);
-    if (p.fmt.rb == 8) k_part_coarse<TYPE, 8, RANGED><<<p.n_cta_part, SORT_THREADS, smem, s>>>(p);
-    else k_part_coarse<TYPE, 16, RANGED><<<p.n_cta_part, SORT_THREADS, smem, s>>>(p);
+cudaError_t coarse_r(const EmitParams& p, cudaStream_t s) {
+    return launch_chained(p.chain, p.fmt.rb == 8 ? k_part_coarse<TYPE, 8, RANGED> : k_part_coarse<TYPE, 16, RANGED>,
+                          p.n_cta_part, SORT_THREADS, coarse_smem<TYPE>(p.fmt.rb), s, p);
 }
 
 template <int TYPE>
 cudaError_t part_coarse_t(const EmitParams& p, cudaStream_t s) {
-    if (ranged(p)) coarse_r<TYPE, true>(p, s);
-    else coarse_r<TYPE, false>(p, s);
-    return cudaGetLastError();
+    return ranged(p) ? coarse_r<TYPE, true>(p, s) : coarse_r<TYPE, false>(p, s);
 }
 
 int coarse_ctas_per_sm(int type) { return type == NN_TET ? SortShape<NN_TET>::CTAS : SortShape<NN_HEX>::CTAS; }
@@ -906,8 +906,7 @@ cudaError_t fine_t(const EmitParams& p, const uint32_t* bstart, int sms, cudaStr
     int occ = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_part_fine<RB, THREADS, RPT, DPT>, THREADS, fs);
     if (e != cudaSuccess) return e;
-    k_part_fine<RB, THREADS, RPT, DPT><<<std::max(1, sms * std::max(occ, 1)), THREADS, fs, s>>>(p, bstart);
-    return cudaGetLastError();
+    return launch_chained(p.chain, k_part_fine<RB, THREADS, RPT, DPT>, std::max(1, sms * std::max(occ, 1)), THREADS, fs, s, p, bstart);
 }
 
 template <int RB>
@@ -964,8 +963,7 @@ cudaError_t launch_slab_count(const EmitParams& p, int shift, int n_slabs, uint3
 cudaError_t launch_offsets(const OffsetsParams& p, cudaStream_t s) {
     const int64_t tiles = (p.n_buckets + OFFSETS_THREADS - 1) / OFFSETS_THREADS;
     if (tiles == 0) return cudaSuccess;
-    k_offsets<<<(unsigned)tiles, OFFSETS_THREADS * (p.n_cta >= 16 ? OFFSETS_SLICES : 1), 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_chained(p.chain, k_offsets, (unsigned)tiles, OFFSETS_THREADS * (p.n_cta >= 16 ? OFFSETS_SLICES : 1), 0, s, p);
 }
 
 cudaError_t set_emit_smem_all(size_t bytes) {

@@ -73,6 +73,8 @@ struct EmitParams {
     uint64_t rec_cap; // records that fit; more only when elem_ptr is invalid
     int32_t* status;
     uint64_t hist_words;  // length of hist (bounds-checked builds)
+    bool chain;           // launched as a chain (launch_chained)
+    bool after_kernel;    // the histogram pass directly follows a kernel of this build
 };
 
 struct BatchHeader;
@@ -92,6 +94,7 @@ struct OffsetsParams {
     uint64_t rec_cap;       // bucket starts are clamped to the record array
     int32_t* status;
     const BatchHeader* hdr; // batches: the bucket count comes from the header
+    bool chain;             // launched as a chain (launch_chained)
 };
 
 // ------------------------------------------------------------------ batches
@@ -172,8 +175,10 @@ struct BucketParams {
     uint64_t nloc_words;    // words of nloc
     uint64_t ngrp;          // entries of grp
     DirectMesh direct;      // single mesh, one bucket per CTA
+    bool chain;             // launched as a chain (launch_chained)
 };
 
+constexpr int64_t CHAIN_RECORDS = 1 << 24;  // incidences up to which a build's kernels are launched as a chain
 constexpr int EMIT_THREADS = 1024;
 constexpr int PART_THREADS = 512;
 constexpr int SORT_THREADS = 256;   // tile-sorted partition passes
@@ -204,6 +209,7 @@ struct CompactParams {
     // buffer lengths, for bounds-checked builds
     uint64_t ntmp_words;     // words of ntmp
     uint64_t nloc_words;     // words of nloc
+    bool chain;              // launched as a chain (launch_chained)
 };
 
 // Element face adjacency (nn_adj.cu).
@@ -248,8 +254,8 @@ cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t s
 size_t bucket_smem_bytes(int sb, int want, int k, int slots, int rb, int list_cap);
 cudaError_t bucket_occupancy(int* blocks, int threads, int imax, size_t smem);
 cudaError_t launch_batch_emit(const BatchTables& bt, uint32_t* bcount, uint32_t* nfc, uint32_t* gcur, uint8_t* rec,
-                              uint64_t* lb_off, uint32_t* ctrl, int grid, int stage, cudaStream_t s,
-                              uint64_t* lb_ns = nullptr);
+                              uint64_t* lb_off, uint32_t* ctrl, int grid, int stage, bool chain,
+                              cudaStream_t s, uint64_t* lb_ns = nullptr);
 int batch_ctas_per_sm();
 cudaError_t set_emit_smem_all(size_t bytes);
 cudaError_t set_bucket_smem_all(size_t bytes);
