@@ -157,10 +157,10 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     // builds), one bucket per SM at most: histogram, offsets and partition are
     // three launches with little to do, while reading the connectivity in
     // every bucket's CTA grows with it.  Graph replays, direct and
-    // partitioned: triangles 3 K incidences 16 and 27 us, 24 K 19 and 30,
-    // quads 16 K 16 and 23, tets 12 K 27 and 35, 41 K 33 and 35, 81 K 38 and
-    // 35, hexes 64 K 27 and 31, mixed 22 K 33 and 37, 43 K 44 and 41; with
-    // more buckets than SMs a second wave doubles the time.
+    // partitioned: triangles 3 K incidences 14 and 25 us, 24 K 18 and 27,
+    // quads 16 K 16 and 21, tets 12 K 26 and 33, 41 K 31 and 33, hexes 11 K 16
+    // and 25, 64 K 27 and 28, mixed 7 K 29 and 35, 22 K 33 and 37; with more
+    // buckets than SMs a second wave made it slower (triangles 59 K 41 and 33).
     const bool tuned = h->sb_override >= 0 || h->part_mode >= 0 || h->hist_chunk_override > 0 ||
                        h->emit_ctas_override > 0 || h->tuning.bucket_ctas_per_sm;
     // (more elements than incidences: an invalid elem_ptr, left to the general path)

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_batch_init(BatchTables bt, ui
 // record while every record had its own; now the shared counters' atomics and
 // the gathered 16-byte stores.  GB300, 24 meshes of 1e3 to 5e5 elements (9.6 M
 // records): histogram 228 -> 24 us, partition 260 -> 148 us, the whole call
-// 787 -> 465 us.  A slice with more buckets than counters has few records per
+// 787 -> 459 us.  A slice with more buckets than counters has few records per
 // bucket to add up, and keeps one global atomic per record.
 __global__ void __launch_bounds__(BATCH_THREADS, 3) k_hist_b(BatchTables bt, uint32_t* bcount, uint32_t* nfc) {
     chain_begin();

@@ -267,8 +267,8 @@ struct Regs {
 // is a launch with next to nothing to do.  What bounds it is the latency of a
 // few dependent steps (triangles 64^2, 128 CTAs: 13 us of a build of 18), so a
 // CTA has as many threads as the registers allow.  Whole builds, graph
-// replays: triangles 64^2 33 -> 18.5 us, hex 21^3 32 -> 27 us; as calls, one
-// after another, triangles 64^2 44 -> 24 us.  scan_elements looks at the elements
+// replays: triangles 64^2 33 -> 18 us, hex 21^3 32 -> 27 us; as calls, one
+// after another, triangles 64^2 44 -> 18 us.  scan_elements looks at the elements
 // [e0, e1): incidences of the nodes [v0, v0 + span) go into the queue (element
 // * 8 + local node), and those of lower nodes are counted (below[0]; below[1]:
 // the repeated-node ones), which gives the bucket's place in the results.

@@ -402,11 +402,10 @@ __host__ __device__ constexpr size_t coarse_smem(int rb) {
 }
 // Tiles of the fine pass: 16 KB of records, 4 to a thread of 256 (8-byte
 // records 8); 2048 records and 512 threads when a coarse region has at least
-// 512 buckets (then a 1024-record tile has two records per bucket, and its one
-// cursor atomic per bucket present comes close to one per two records: L2
-// atomics, about 40 G/s, bind the pass).  hex 257^3 and mixed 257^3: 256
-// threads of 8 records 943 and 1503 us, 512 of 8 857 and 1366 us, 512 of 4 807
-// and 1285 us.
+// 512 buckets: a 1024-record tile would have two records per bucket, and its
+// one cursor atomic per bucket present come close to one per two records.
+// hex 257^3 and mixed 257^3: 256 threads of 8 records 943 and 1503 us (16 warps
+// per SM), 512 of 8 857 and 1366 us, 512 of 4 807 and 1285 us.
 constexpr int FINE_WIDE_DIGITS = 512;
 __host__ __device__ constexpr int fine_threads(int nd) { return nd >= FINE_WIDE_DIGITS ? 512 : 256; }
 __host__ __device__ constexpr int fine_rpt(int nd, int rb) { return nd < FINE_WIDE_DIGITS && rb == 8 ? 8 : 4; }
