@@ -338,6 +338,12 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     auto mark = [&](int i) {
         if (prof) prof_mark(h, i, s);
     };
+    // A direct build has no offsets scan and no node-row scan (a single mesh's
+    // rows are placed by sums), so it has no lookback words to clear.  It is
+    // always the whole mesh, hence never one of several chunks: those place
+    // their rows by the scan and begin with a memset, which a kernel launched
+    // as a dependent one may not follow.
+    if (p.direct && base) return NN_ERR_ARG;
     const size_t zero = p.direct ? p.off_ctrl : p.zero_begin;
     // (the chunks of a chunked build keep one status word)
     if ((base ? cudaMemsetAsync(w + zero, 0, p.zero_end - zero, s)
@@ -1089,11 +1095,15 @@ nn_status nn_neighbors_chunked(nn_handle* h, const nn_mesh* mesh, int want, cons
         return NN_OK;
     }
     uint8_t* cw = w + ALIGN;
+    // a chunk that is the whole mesh is a single build, with no offsets to run on
+    const bool single = n_chunks == 1;
     for (int c = 0; c < n_chunks; ++c) {
         Plan p;
         make_plan_range(h, mesh, want, chunks[c].node_lo, chunks[c].node_hi - chunks[c].node_lo, chunks[c].records, &p);
-        if ((st = enqueue(h, mesh, p, nodes, elems, cw, ws_bytes - ALIGN, base, d_status, false, s)) != NN_OK)
+        if ((st = enqueue(h, mesh, p, nodes, elems, cw, ws_bytes - ALIGN, single ? nullptr : base, d_status, false, s)) !=
+            NN_OK)
             return st;
+        if (single) break;
         // (the chunk's totals end its two scans)
         const uint32_t* etot = (want & NN_WANT_ELEMS) ? reinterpret_cast<const uint32_t*>(cw + p.off_estart) + p.B : nullptr;
         const uint64_t* ntot = (want & NN_WANT_NODES) ? reinterpret_cast<const uint64_t*>(cw + p.off_nstart) + p.B * p.groups : nullptr;
