@@ -220,7 +220,11 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
         per_sm = 1;
     p.bucket_grid = (int)std::min<int64_t>(p.B, (int64_t)h->sms * per_sm);
 
-    if (direct && f.cshift == 0 && p.B <= h->sms && p.bucket_smem + DIRECT_QUEUE * 4 <= h->bucket_smem) {
+    // (few enough groups that their rows are placed by sums: wide buckets, a
+    // tuning, of very many nodes have more, and the scan over them is given no
+    // cleared words by a direct build)
+    if (direct && f.cshift == 0 && p.B <= h->sms && p.B * p.groups <= NODE_SUM_GROUPS &&
+        p.bucket_smem + DIRECT_QUEUE * 4 <= h->bucket_smem) {
         p.direct = true;
         p.queue_cap = DIRECT_QUEUE;
     }
