@@ -180,7 +180,6 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     if (h->sb_override >= SB_MIN && h->sb_override <= SB_MAX) sb = h->sb_override;
     // wider buckets than shared memory holds (a tuning, a test): fewer slots,
     // then fewer nodes
-    constexpr int SLOTS_MIN = 4;
     while (sb > SB_MIN && need(sb, SLOTS_MIN) > h->bucket_smem) --sb;
     while (nbk(sb) > B_max && sb < SB_MAX) ++sb;
     if (nbk(sb) > B_max || need(sb, SLOTS_MIN) > h->bucket_smem) return NN_ERR_ARG;

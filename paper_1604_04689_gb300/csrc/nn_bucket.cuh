@@ -232,8 +232,12 @@ struct BucketMeta {
 };
 
 // Words of a node's neighbour column: its slots, and room for a triangle fan
-// of 22 around a node whose slots are few.
-__host__ __device__ constexpr int ncol_of(int k, int slots) { return k * slots > 24 ? k * slots : 24; }
+// of 22 around a node whose slots are few.  (Of 14 with the fewest slots: that
+// is what buckets of 2048 nodes have room for, which meshes of more than 2^30
+// nodes need to stay within 2^20 buckets.)
+__host__ __device__ constexpr int ncol_of(int k, int slots) {
+    return slots <= SLOTS_MIN ? 16 : (k * slots > 24 ? k * slots : 24);
+}
 // Words of a node's element column.  Without a neighbour column the rows are
 // put together here, where listed records add to the slots.
 __host__ __device__ constexpr int ecol_of(int want, int slots) {

@@ -184,6 +184,7 @@ constexpr int PART_THREADS = 512;
 constexpr int SORT_THREADS = 256;   // tile-sorted partition passes
 constexpr int OFFSETS_THREADS = 128;  // buckets per tile of the offsets scan
 constexpr int OFFSETS_SLICES = 8;     // slices of its histogram rows summed side by side
+constexpr int SLOTS_MIN = 4;  // fewest slots of a node in the bucket pass
 constexpr int NODE_SCAN_TILE = 512;  // groups of 32 nodes per tile of the node-row placement's scan
 
 // groups up to which the placement adds up a group's predecessors itself (16
