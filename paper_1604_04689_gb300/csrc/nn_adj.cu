@@ -605,7 +605,8 @@ template <int TYPE>
 void match_and_write(const AdjParams& p, int grid, int sms, cudaStream_t s) {
     constexpr int NODES = ADJ_THREADS / AdjShape<TYPE>::G;  // nodes of a CTA at a time
     const int64_t blocks = (p.n_nodes + NODES - 1) / NODES;
-    k_adj_match<TYPE><<<(unsigned)(blocks < (int64_t)sms * 16 ? blocks : (int64_t)sms * 16), ADJ_THREADS, 0, s>>>(p);
+    if (blocks > 0)  // (without nodes every element is invalid and has an empty row)
+        k_adj_match<TYPE><<<(unsigned)(blocks < (int64_t)sms * 16 ? blocks : (int64_t)sms * 16), ADJ_THREADS, 0, s>>>(p);
     count_scan_write<TYPE>(p, grid, s);
 }
 
