@@ -131,24 +131,9 @@ __device__ inline void warp_bitonic_sort(uint32_t* a, uint32_t n) {
     }
 }
 
-// A record of the bucket being built by its whole CTA.  In a direct build the
-// CTA has written it itself (no read-only load).
-template <int RB, bool DIRECT>
-__device__ __forceinline__ Rec own_rec(const uint8_t* base, uint64_t pos) {
-    if constexpr (!DIRECT) {
-        return load_rec<RB>(base, pos);
-    } else if constexpr (RB == 8) {
-        const uint2 v = __ldcg(reinterpret_cast<const uint2*>(base) + pos);
-        return Rec{v.x, v.y, 0u, 0u};
-    } else {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(base) + pos);
-        return Rec{v.x, v.y, v.z, v.w};
-    }
-}
-
 // The element ids of a node's c records (a repeated node's record adds
 // none), collected by its whole warp into row[0..ec) and sorted there.
-template <int RB, int K, bool DIRECT>
+template <int RB, int K>
 __device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, const uint32_t* grp, uint32_t c,
                                            uint32_t* row, uint32_t ec) {
     const uint32_t lane = threadIdx.x & 31;
@@ -158,7 +143,7 @@ __device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, c
         bool keep = false;
         uint32_t e = 0;
         if (s < c) {
-            const Rec x = own_rec<RB, DIRECT>(rp, grp[s]);
+            const Rec x = take_rec<RB>(rp, grp[s]);
             keep = !((rec_side<RB, K>(f, x) >> f.off_nf) & 1u);
             e = rec_elem<RB>(f, x);
         }
@@ -172,13 +157,13 @@ __device__ __noinline__ void warp_elem_row(const RecFmt& f, const uint8_t* rp, c
 
 // The distinct neighbours of a node's c records, collected by its whole warp
 // into a[0 .. K c): sorted, the first of every run kept.  Returns their count.
-template <int RB, int K, bool DIRECT>
+template <int RB, int K>
 __device__ __noinline__ uint32_t warp_node_row(const RecFmt& f, const uint8_t* rp, const uint32_t* grp, uint32_t c,
                                                uint32_t* a) {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t nc = (uint64_t)K * c;
     for (uint32_t s = lane; s < c; s += 32) {
-        const Rec x = own_rec<RB, DIRECT>(rp, grp[s]);
+        const Rec x = take_rec<RB>(rp, grp[s]);
 #pragma unroll
         for (int j = 0; j < K; ++j) a[(uint64_t)s * K + j] = rec_nbr<RB>(f, x, j);
     }
@@ -579,7 +564,7 @@ __global__ void __launch_bounds__(DIRECT ? direct_threads(IMAX) : 256, DIRECT ? 
             Rec x[U];
 #pragma unroll
             for (int q = 0; q < U; ++q)
-                if (rb + q * T + tid < R) x[q] = load_rec<RB>(rp, rb + q * T + tid);
+                if (rb + q * T + tid < R) x[q] = take_rec<RB>(rp, rb + q * T + tid);
 #pragma unroll
             for (int q = 0; q < U; ++q) {
                 if (rb + q * T + tid >= R) break;
@@ -799,7 +784,7 @@ __global__ void __launch_bounds__(DIRECT ? direct_threads(IMAX) : 256, DIRECT ? 
         const bool ok = sh_spill[1] >= need;
         uint32_t* const grp = p.spill + sh_spill[0];
         for (uint32_t r = tid; ok && r < R; r += T)
-            grp[atomicAdd(&cursor[rec_side<RB, K>(f, own_rec<RB, DIRECT>(rp, r)) & vmask], 1u)] = r;
+            grp[atomicAdd(&cursor[rec_side<RB, K>(f, take_rec<RB>(rp, r)) & vmask], 1u)] = r;
         __syncthreads();
         uint32_t* const scratch = table + 2 * NB + warp * scratch_words;
         for (int g = warp; g < GP; g += W) {
@@ -813,7 +798,7 @@ __global__ void __launch_bounds__(DIRECT ? direct_threads(IMAX) : 256, DIRECT ? 
                 if (want_e) {
                     if (lane == 0 && NN_IN(v0 + l, N + 1, status)) sh_out.rp_e[v0 + l] = (int64_t)(M.ge + eoff[l]);
                     if (ok && e_ok && c) {
-                        warp_elem_row<RB, K, DIRECT>(sh_fmt, rp, grp + o, c, a, ec);
+                        warp_elem_row<RB, K>(sh_fmt, rp, grp + o, c, a, ec);
                         for (uint32_t k = lane; k < ec; k += 32) sh_out.col_e[M.ge + eoff[l] + k] = (int32_t)a[k];
                         __syncwarp();
                     }
@@ -821,7 +806,7 @@ __global__ void __launch_bounds__(DIRECT ? direct_threads(IMAX) : 256, DIRECT ? 
                 if (want_n) {
                     uint32_t u = 0;
                     if (ok && c) {
-                        u = warp_node_row<RB, K, DIRECT>(sh_fmt, rp, grp + o, c, a);
+                        u = warp_node_row<RB, K>(sh_fmt, rp, grp + o, c, a);
                         const size_t d = (size_t)K * (M.r0 + pr) + run;
                         if (u == 0 || NN_IN(d + u - 1, p.ntmp_words, status))
                             for (uint32_t k = lane; k < u; k += 32) p.ntmp[d + k] = a[k];

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_node_scan(CompactParams p) {
 // totals of the groups before them itself, which for a few thousand groups
 // costs less than the scan's launch.
 template <bool SUM>
-__global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
+__global__ void __launch_bounds__(COPY_THREADS, 8) k_node_copy(CompactParams p) {
     chain_begin();
     const bool batched = p.batch.hdr != nullptr;
     const int64_t B = batched ? p.batch.hdr->n_buckets : p.n_buckets;
@@ -73,10 +73,10 @@ __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
         __shared__ uint64_t sh_scan[33];
         const int64_t first = (int64_t)blockIdx.x * (COPY_THREADS / 32), mine = first + (threadIdx.x >> 5);
         uint64_t x = 0, total;
-        for (int64_t i = threadIdx.x; i < first; i += COPY_THREADS) x += __ldg(&p.grp[i].y);
+        for (int64_t i = threadIdx.x; i < first; i += COPY_THREADS) x += p.grp[i].y;
         block_excl_scan(x, &total, sh_scan);
         before = total;
-        for (int64_t i = first; i < mine && i < n; ++i) before += __ldg(&p.grp[i].y);
+        for (int64_t i = first; i < mine && i < n; ++i) before += p.grp[i].y;
     }
     for (int64_t gi = (int64_t)blockIdx.x * (COPY_THREADS / 32) + (threadIdx.x >> 5); gi < n; gi += warps) {
         const int64_t b = gi / GP;
@@ -116,7 +116,22 @@ __global__ void __launch_bounds__(COPY_THREADS) k_node_copy(CompactParams p) {
         const uint32_t* src = p.ntmp + (size_t)K * g.x;
         int32_t* dst = col + gn;
         if (!NN_IN((size_t)K * g.x + (g.y ? g.y - 1 : 0), p.ntmp_words + (g.y ? 0 : 1), status)) continue;
-        for (uint32_t i = lane; i < g.y; i += 32) dst[i] = (int32_t)__ldg(src + i);
+        // (four loads in flight: ordinary ones may not pass the stores before them)
+        uint32_t i = lane;
+        for (; i + 96 < g.y; i += 128) {
+            const uint32_t a = src[i], b = src[i + 32], c = src[i + 64], d = src[i + 96];
+            dst[i] = (int32_t)a;
+            dst[i + 32] = (int32_t)b;
+            dst[i + 64] = (int32_t)c;
+            dst[i + 96] = (int32_t)d;
+        }
+        uint32_t x[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (i + 32 * k < g.y) x[k] = src[i + 32 * k];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (i + 32 * k < g.y) dst[i + 32 * k] = (int32_t)x[k];
     }
 }
 

@@ -35,7 +35,9 @@ __device__ __forceinline__ bool in_bounds(uint64_t i, uint64_t n, int32_t* st) {
 // there is room for them.  Each kernel that is launched so begins with
 // chain_begin(): it waits until the kernel before it is complete and its
 // writes are visible, then lets the next one be set up.  (A kernel waits for
-// its predecessor alone, which has waited for its own.)  Builds
+// its predecessor alone, which has waited for its own.)  What earlier kernels
+// of the sequence have written is read with ordinary loads; __ldg is for the
+// caller's mesh, which does not change while any of them is there.  Builds
 // of up to CHAIN_RECORDS incidences are launched so: between kernels of a few
 // microseconds the launches are a good part of the time (one call after
 // another: 1.76 M triangles 174 -> 165 us, 1 M quads' node rows 138 -> 124 us,
@@ -265,6 +267,9 @@ __device__ __forceinline__ void put_rec(uint8_t* base, uint64_t pos, const Rec& 
     if constexpr (RB == 8) reinterpret_cast<uint2*>(base)[pos] = make_uint2(r.x, r.y);
     else reinterpret_cast<uint4*>(base)[pos] = make_uint4(r.x, r.y, r.z, r.w);
 }
+// Shared memory, or records in global memory.  Never a read-only load (__ldg):
+// a kernel of a chain (chain_begin) is there before the one that writes them
+// is done, and only ordinary loads are sure to stay behind its wait.
 template <int RB>
 __device__ __forceinline__ Rec take_rec(const uint8_t* base, uint64_t pos) {
     if constexpr (RB == 8) {
@@ -275,18 +280,6 @@ __device__ __forceinline__ Rec take_rec(const uint8_t* base, uint64_t pos) {
         return Rec{v.x, v.y, v.z, v.w};
     }
 }
-// Read-only global memory (written by an earlier kernel).
-template <int RB>
-__device__ __forceinline__ Rec load_rec(const uint8_t* base, uint64_t pos) {
-    if constexpr (RB == 8) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2*>(base) + pos);
-        return Rec{v.x, v.y, 0u, 0u};
-    } else {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(base) + pos);
-        return Rec{v.x, v.y, v.z, v.w};
-    }
-}
-
 // ------------------------------------------------ element local edge tables
 // Edge-neighbors of local node i (the other end of each local edge at i).
 // tri: the two others; quad: the two cyclic neighbours; tet: the three others;
