@@ -75,6 +75,7 @@ struct Plan {
     bool direct = false;                      // no partition: every bucket's CTA reads the whole connectivity
     int queue_cap = 0;                        // ... incidences it queues at a time
     size_t bucket_smem = 0;
+    RestShape rest{};         // the bucket pass's second launch
 };
 
 nn_status check_mesh(const nn_mesh* m) {
@@ -117,6 +118,21 @@ bool record_format(int sb, int want, int k, int64_t T, int64_t N, int cshift, in
     f.sh0 = std::min(31, 3 * (32 - f.nb));
     *out = f;
     return true;
+}
+
+// Second launch of the bucket pass (nn_bucket.cuh): as many of 32 slots as two
+// CTAs per SM leave room for, SLOTS_MIN at least, and a list of 512 records.
+RestShape rest_shape(const nn_handle* h, int sb, int want, int k, int rb, int64_t buckets) {
+    RestShape r{SLOTS_MIN, 512, sb >= 8 ? 256 : 128, 1, 0};
+    const int per_sm = sb >= 8 ? 2 : 4;  // by registers
+    auto need = [&](int slots) { return bucket_smem_bytes(sb, want, k, slots, rb, r.list_cap); };
+    const size_t room = std::min(h->bucket_smem, h->smem_per_sm / 2 - 2048);
+    while (r.list_cap > 32 && need(SLOTS_MIN) > h->bucket_smem) r.list_cap -= 16;
+    while (r.slots < 32 && need(r.slots + 1) <= room) ++r.slots;
+    r.smem = need(r.slots);
+    const size_t fit = h->smem_per_sm / (r.smem + 2048);
+    r.grid = (int)std::min<int64_t>(buckets, (int64_t)h->sms * std::max<size_t>(1, std::min<size_t>(fit, per_sm)));
+    return r;
 }
 
 // Plan of a build over the nodes [lo, lo + span) of mesh m, which have
@@ -186,6 +202,14 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     p.slots = SLOTS_MIN;
     while (p.slots < want_slots && need(sb, p.slots + 1) <= h->bucket_smem) ++p.slots;
     p.list_cap = list_of(sb);
+    // the list takes what the resident CTAs leave over, up to 512 records:
+    // 3-d Delaunay meshes (27 records per node, some of 40) list 320 of a
+    // bucket of 128 nodes
+    const int by_regs = p.imax == 8 ? 1024 : (p.imax == 16 ? 768 : 512);
+    const size_t base_smem = bucket_smem_bytes(sb, want, p.k, p.slots, 16, p.list_cap);
+    const size_t resident = std::max<size_t>(1, std::min<size_t>((size_t)(by_regs / p.bucket_threads), h->smem_per_sm / (base_smem + 1536)));
+    const size_t per_cta = std::min(h->bucket_smem, h->smem_per_sm / resident - 1536);
+    while (p.list_cap < 512 && bucket_smem_bytes(sb, want, p.k, p.slots, 16, p.list_cap + 16) <= per_cta) p.list_cap += 16;
     p.groups = sb < 5 ? 1 : 1 << (sb - 5);
     p.B = nbk(sb);
 
@@ -222,6 +246,7 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     // (few enough groups that their rows are placed by sums: wide buckets, a
     // tuning, of very many nodes have more, and the scan over them is given no
     // cleared words by a direct build)
+    p.rest = rest_shape(h, sb, want, p.k, f.rb, p.B);
     if (direct && f.cshift == 0 && p.B <= h->sms && p.B * p.groups <= NODE_SUM_GROUPS &&
         p.bucket_smem + DIRECT_QUEUE * 4 <= h->bucket_smem) {
         p.direct = true;
@@ -260,8 +285,8 @@ nn_status make_plan_range(const nn_handle* h, const nn_mesh* m, int want, int64_
     p.zero_end = o;
     p.off_spill = o;
     p.ws_min = o;
-    // spill area: buckets built by a whole CTA group their record indices and
-    // sort long rows there (16 MB and 8 bytes per record covers the odd node
+    // spill area: the record indices of hard nodes (nn_bucket.cuh) are grouped
+    // there, and long element rows sorted (16 MB and 8 bytes per record covers the odd node
     // of very high valence); a plan whose typical bucket has too few slots (a
     // tuning that widens the buckets) gets room for all of them
     size_t spill = ((size_t)16 << 20) + (size_t)p.n_conn * 8;
@@ -426,6 +451,10 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
     bp.imax = p.imax;
     bp.slots = p.slots;
     bp.list_cap = p.list_cap;
+    bp.rest = reinterpret_cast<uint32_t*>(w + p.off_gcur);  // (the partition's cursors, dead by now)
+    bp.rest_count = ctrl + 5;
+    bp.rest_ticket = ctrl + 6;
+    bp.rest_cap = (uint64_t)p.B;
     bp.ntmp = reinterpret_cast<uint32_t*>(w + p.off_ntmp);
     bp.grp = reinterpret_cast<uint2*>(w + p.off_grp);
     bp.nloc = reinterpret_cast<uint32_t*>(w + p.off_nloc);
@@ -452,8 +481,8 @@ nn_status enqueue(nn_handle* h, const nn_mesh* m, const Plan& p, nn_csr* nodes, 
         mark(4);
     }
     mark(5);
-    if (p.direct ? launch_bucket(bp, (int)p.B, p.bucket_threads, p.bucket_smem + (size_t)p.queue_cap * 4, s) != cudaSuccess
-                 : launch_bucket(bp, p.bucket_grid, p.bucket_threads, p.bucket_smem, s) != cudaSuccess)
+    if (p.direct ? launch_bucket(bp, (int)p.B, p.bucket_threads, p.bucket_smem + (size_t)p.queue_cap * 4, p.rest, s) != cudaSuccess
+                 : launch_bucket(bp, p.bucket_grid, p.bucket_threads, p.bucket_smem, p.rest, s) != cudaSuccess)
         return NN_ERR_CUDA;
     mark(6);
     if (want & NN_WANT_NODES) {
@@ -495,6 +524,7 @@ struct BatchPlan {
     size_t off_bcount = 0, off_bstart = 0, off_gcur = 0, off_rec = 0, off_lb_off = 0, off_ctrl = 0, off_spill = 0, ws_min = 0, ws_rec = 0, off_nfc = 0,
            off_estart = 0, off_ntmp = 0, off_grp = 0, off_nloc = 0, off_nstart = 0, off_lb_ns = 0;
     size_t bucket_smem = 0;
+    RestShape rest{};
     int bucket_grid = 0, emit_grid = 0, bucket_threads = 128;
     int64_t tiles_cap = 0;
 };
@@ -524,6 +554,7 @@ nn_status batch_plan(const nn_handle* h, const nn_batch_caps* c, BatchPlan* out)
     int per_sm = 1;
     if (bucket_occupancy(&per_sm, p.bucket_threads, 32, p.bucket_smem) != cudaSuccess || per_sm < 1) per_sm = 1;
     p.bucket_grid = h->sms * per_sm;
+    p.rest = rest_shape(h, p.sb, c->want, 3, 16, p.B_cap);
     size_t o = p.table_bytes;
     p.off_bcount = o; o = align_up(o + (size_t)p.B_cap * 4);
     p.off_nfc = o; o = align_up(o + (size_t)p.B_cap * 4);
@@ -676,6 +707,10 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     kp.chain = chain;
     kp.slots = BATCH_SLOTS;
     kp.list_cap = BATCH_LIST;
+    kp.rest = gcur;  // (dead after the partition)
+    kp.rest_count = ctrl + 5;
+    kp.rest_ticket = ctrl + 6;
+    kp.rest_cap = (uint64_t)bp.B_cap;
     kp.ntmp = reinterpret_cast<uint32_t*>(w + bp.off_ntmp);
     kp.grp = reinterpret_cast<uint2*>(w + bp.off_grp);
     kp.nloc = reinterpret_cast<uint32_t*>(w + bp.off_nloc);
@@ -683,7 +718,7 @@ nn_status batch_launch(nn_handle* h, const nn_batch_caps* c, const void* staging
     kp.ntmp_words = (c->want & NN_WANT_NODES) ? 3 * (uint64_t)c->max_conn + 4 : 0;
     kp.nloc_words = (c->want & NN_WANT_NODES) ? (uint64_t)bp.B_cap << bp.sb : 0;
     kp.ngrp = (c->want & NN_WANT_NODES) ? (uint64_t)bp.B_cap * bp.groups : 0;
-    if (launch_bucket(kp, bp.bucket_grid, bp.bucket_threads, bp.bucket_smem, s) != cudaSuccess) return NN_ERR_CUDA;
+    if (launch_bucket(kp, bp.bucket_grid, bp.bucket_threads, bp.bucket_smem, bp.rest, s) != cudaSuccess) return NN_ERR_CUDA;
     if (c->want & NN_WANT_NODES) {
         CompactParams cp{};
         cp.n_groups_cap = bp.B_cap * bp.groups;
@@ -819,8 +854,8 @@ nn_status nn_plan_info(nn_handle* h, const nn_mesh* mesh, int want, int64_t* inf
     Plan p;
     nn_status st = make_plan(h, mesh, want, &p);
     if (st != NN_OK) return st;
-    // initialization, histogram, offsets and partition unless direct, buckets, placement of node rows
-    const int64_t kernels = 2 + (p.direct ? 0 : 3 + (p.fmt.cshift > 0)) +
+    // initialization, histogram, offsets and partition unless direct, buckets (twice unless direct), placement of node rows
+    const int64_t kernels = 2 + (p.direct ? 0 : 4 + (p.fmt.cshift > 0)) +
                             (want & NN_WANT_NODES ? (p.B * p.groups <= NODE_SUM_GROUPS ? 1 : 2) : 0);
     const int64_t v[10] = {p.fmt.sb, p.B, p.G, p.fmt.rb, (int64_t)p.ws_min, p.bucket_grid, p.bucket_threads,
                            (int64_t)p.bucket_smem, p.fmt.cshift, p.N > 0 ? kernels : 0};

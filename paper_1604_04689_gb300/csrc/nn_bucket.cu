@@ -7,9 +7,11 @@ namespace nn {
 cudaError_t launch_bucket_16(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_bucket_32(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_bucket_direct(const BucketParams& p, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_bucket_rest(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
 cudaError_t set_bucket_smem_16(size_t bytes);
 cudaError_t set_bucket_smem_32(size_t bytes);
 cudaError_t set_bucket_smem_direct(size_t bytes);
+cudaError_t set_bucket_smem_rest(size_t bytes);
 cudaError_t bucket_occupancy_16(int* blocks, int threads, size_t smem);
 cudaError_t bucket_occupancy_32(int* blocks, int threads, size_t smem);
 
@@ -18,12 +20,26 @@ size_t bucket_smem_bytes(int sb, int want, int k, int slots, int rb, int list_ca
     return 24 * nb + list_bytes(rb, list_cap) + groups * 32 * (size_t)col_words(want, k, slots) * 4;
 }
 
-cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s) {
-    if (grid <= 0) return cudaSuccess;
-    if (p.direct.conn) return launch_bucket_direct(p, grid, smem, s);
+namespace {
+
+cudaError_t launch_plain(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s) {
     if (p.imax == 8) return launch_bucket_t<8>(p, grid, threads, smem, s);
     if (p.imax == 16) return launch_bucket_16(p, grid, threads, smem, s);
     return launch_bucket_32(p, grid, threads, smem, s);
+}
+
+}  // namespace
+
+cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, const RestShape& rest, cudaStream_t s) {
+    if (grid <= 0) return cudaSuccess;
+    if (p.direct.conn) return launch_bucket_direct(p, grid, smem, s);
+    const cudaError_t e = launch_plain(p, grid, threads, smem, s);
+    if (e != cudaSuccess) return e;
+    BucketParams q = p;
+    q.slots = rest.slots;
+    q.list_cap = rest.list_cap;
+    q.ticket = p.rest_ticket;
+    return launch_bucket_rest(q, rest.grid, rest.threads, rest.smem, s);
 }
 
 cudaError_t set_bucket_smem_all(size_t bytes) {
@@ -31,6 +47,7 @@ cudaError_t set_bucket_smem_all(size_t bytes) {
     if (e == cudaSuccess) e = set_bucket_smem_16(bytes);
     if (e == cudaSuccess) e = set_bucket_smem_32(bytes);
     if (e == cudaSuccess) e = set_bucket_smem_direct(bytes);
+    if (e == cudaSuccess) e = set_bucket_smem_rest(bytes);
     return e;
 }
 

@@ -166,6 +166,10 @@ struct BucketParams {
     int32_t imax;           // 8, 16 or 32: the variant by its register arrays
     int32_t slots;          // places per node in the shared-memory table (<= imax)
     int32_t list_cap;       // records beyond their node's slots that a bucket may have
+    uint32_t* rest;         // buckets that the first launch leaves to a second one (room for all)
+    uint32_t* rest_count;   // ... how many
+    uint32_t* rest_ticket;
+    uint64_t rest_cap;      // words of rest
     BatchTables batch;      // batch.hdr != nullptr: format, bucket count and meshes come from the tables
     const int32_t* batch_err;  // batches: status of the shared offsets scan, copied to every mesh
     const int64_t* base;    // chunked builds: {element-CSR, node-CSR} entries of the earlier chunks (else nullptr)
@@ -176,6 +180,12 @@ struct BucketParams {
     uint64_t ngrp;          // entries of grp
     DirectMesh direct;      // single mesh, one bucket per CTA
     bool chain;             // launched as a chain (launch_chained)
+};
+
+// Shape of the bucket pass's second launch.
+struct RestShape {
+    int slots, list_cap, threads, grid;
+    size_t smem;
 };
 
 constexpr int64_t CHAIN_RECORDS = 1 << 24;  // incidences up to which a build's kernels are launched as a chain
@@ -250,7 +260,7 @@ cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s);
 int coarse_ctas_per_sm(int type);
 cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s);
 cudaError_t launch_offsets(const OffsetsParams& p, cudaStream_t s);
-cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, cudaStream_t s);
+cudaError_t launch_bucket(const BucketParams& p, int grid, int threads, size_t smem, const RestShape& rest, cudaStream_t s);
 // dynamic shared memory of the bucket kernel for buckets of 2^sb nodes
 size_t bucket_smem_bytes(int sb, int want, int k, int slots, int rb, int list_cap);
 cudaError_t bucket_occupancy(int* blocks, int threads, int imax, size_t smem);
