@@ -148,7 +148,13 @@ __device__ __forceinline__ void for_each_neighbour(const AdjParams& p, int64_t e
 // table per warp.  Hexes and quads also ask whether a face's nodes lie in an
 // element whose face it is not, and compare pairs in groups of 8.
 constexpr int FACE_HASH_BITS = 7;
-constexpr int ADJ_LONG = 64;  // longest node row matched here; elements around a longer one are flagged
+// Longest node row matched here; elements around a longer one are flagged
+// without a look at them.  Rows longer than a group's are matched by the whole
+// warp (an element per lane, the others by shuffles); they used to be by the
+// group, against nodes read from memory.  Whole call, before and now: random
+// hexes with 8 elements a node 1040 -> 557 us, random quads 510 -> 325, Delaunay
+// triangles 283 -> 232, a sphere with poles of 1000 781 -> 744.
+constexpr int ADJ_LONG = 64;
 
 template <int TYPE>
 struct AdjShape;
@@ -277,6 +283,18 @@ struct AdjFrame {
             return (in[0] && in[1] && in[2] ? 1u : 0u) | (in[0] && in[3] && in[4] ? 2u : 0u) |
                    (in[1] && in[3] && in[5] ? 4u : 0u);
     }
+    // hex: whether two of the three nodes next to v, which every face at v has,
+    // are in y (else: true)
+    __device__ __forceinline__ bool may_share(const int32_t* y) const {
+        if constexpr (TYPE == NN_HEX) {
+            int n = 0;
+#pragma unroll
+            for (int i = 0; i < S::Q; ++i) n += (q[0] == y[i]) + (q[1] == y[i]) + (q[3] == y[i]);
+            return n >= 2;
+        } else {
+            return true;
+        }
+    }
     // whether face f at v is, as far as a look at the frames shows, a face of
     // y too (simplices: always; a false "no" only costs the slow path)
     __device__ __forceinline__ bool also_face_of(int f, const int32_t* y) const {
@@ -294,10 +312,11 @@ struct AdjFrame {
     }
 };
 
-// One node per group of G lanes, one element of its row per lane (rows of
-// more than G elements: several rounds, the others read from memory).
+// One node per group of G lanes, one element of its row per lane; rows of more
+// than G elements by the whole warp.  (Triangles: 5 CTAs per SM; left alone, the
+// compiler spills for a sixth, 1500^2 nodes 560 -> 575 us.)
 template <int TYPE>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_match(AdjParams p) {
+__global__ void __launch_bounds__(ADJ_THREADS, TYPE == NN_TRI ? 5 : 0) k_adj_match(AdjParams p) {
     using S = AdjShape<TYPE>;
     constexpr int G = S::G, PER = 32 / G;
     __shared__ __align__(16) uint32_t sh_head[TYPE == NN_TET ? ADJ_THREADS / 32 : 1][1 << FACE_HASH_BITS];
@@ -409,25 +428,45 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_match(AdjParams p) {
             }
         }
         if (ok == 1) settle(x, v, e, r);
-        if (n <= G) continue;
-        for (int64_t i = gl; i < n; i += G) {
-            const int32_t ei = __ldg(p.ne_col + cur + i);
-            AdjFrame<TYPE> xi{};
-            const int oki = xi.load(p, ei, v);
-            if (!oki) continue;
-            if (n > ADJ_LONG) {
-                p.cplx[ei] = 1;
+        // longer rows, one after another by the whole warp: 32 elements at a
+        // time against 32 at a time
+        for (unsigned m = __ballot_sync(0xffffffffu, gl == 0 && n > G); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const int64_t nl = __shfl_sync(0xffffffffu, n, src), at = __shfl_sync(0xffffffffu, cur, src);
+            const int32_t vl = __shfl_sync(0xffffffffu, v, src);
+            if (nl > ADJ_LONG) {
+                for (int64_t i = lane; i < nl; i += 32) {
+                    const int32_t ei = __ldg(p.ne_col + at + i);
+                    if (ei >= 0 && ei < p.n_elems) p.cplx[ei] = 1;
+                }
                 continue;
             }
-            Found ri{};
-            for (int64_t j = 0; j < n; ++j) {
-                const int32_t ey = __ldg(p.ne_col + cur + j);
-                AdjFrame<TYPE> y{};
-                const int oky = y.load(p, ey, v);
-                if (oky == 2) p.cplx[ei] = 1;
-                if (oky && ey != ei) compare(xi, v, ey, y.q, ri);
+            for (int64_t i0 = 0; i0 < nl; i0 += 32) {
+                const int32_t ei = i0 + lane < nl ? __ldg(p.ne_col + at + i0 + lane) : -1;
+                AdjFrame<TYPE> xi{};
+                const int oki = xi.load(p, ei, vl);
+                Found ri{};
+                for (int64_t j0 = 0; j0 < nl; j0 += 32) {
+                    AdjFrame<TYPE> y = xi;
+                    int32_t ej = ei;
+                    int oky = oki;
+                    if (j0 != i0) {
+                        ej = j0 + lane < nl ? __ldg(p.ne_col + at + j0 + lane) : -1;
+                        oky = y.load(p, ej, vl);
+                    }
+                    // a repeated node: the elements around this node take the slow path
+                    if (__any_sync(0xffffffffu, oky == 2) && oki) p.cplx[ei] = 1;
+                    const int32_t id_j = oky ? ej : -1;
+                    for (int j = 0; j < 32 && j0 + j < nl; ++j) {
+                        const int32_t ey = __shfl_sync(0xffffffffu, id_j, j);
+                        int32_t yq[S::Q];
+#pragma unroll
+                        for (int k = 0; k < S::Q; ++k) yq[k] = __shfl_sync(0xffffffffu, y.q[k], j);
+                        if (oki && ey >= 0 && ey != ei && xi.may_share(yq)) compare(xi, vl, ey, yq, ri);
+                    }
+                }
+                if (oki == 1) settle(xi, vl, ei, ri);
             }
-            if (oki == 1) settle(xi, v, ei, ri);
         }
     }
 }
