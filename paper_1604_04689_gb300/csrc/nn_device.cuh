@@ -176,23 +176,6 @@ __device__ inline uint64_t block_excl_scan(uint64_t x, uint64_t* total, uint64_t
     return r;
 }
 
-// Exclusive scan in place of a shared array of n 64-bit values; returns the sum.
-__device__ inline uint64_t smem_array_excl_scan(uint64_t* a, int n, uint64_t* sh) {
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int lo = min(n, (int)threadIdx.x * per), hi = min(n, lo + per);
-    uint64_t s = 0;
-    for (int i = lo; i < hi; ++i) s += a[i];
-    uint64_t total;
-    uint64_t run = block_excl_scan(s, &total, sh);
-    for (int i = lo; i < hi; ++i) {
-        uint64_t t = a[i];
-        a[i] = run;
-        run += t;
-    }
-    __syncthreads();
-    return total;
-}
-
 // --------------------------------------------------------------- records
 // (the layout is described at RecFmt; 8-byte records use x and y)
 struct Rec {

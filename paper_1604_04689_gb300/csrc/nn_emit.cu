@@ -936,12 +936,6 @@ cudaError_t set_fine_smem() {
     return e;
 }
 
-cudaError_t launch_part_sorted(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s) {
-    cudaError_t e = launch_part_coarse(p, s);
-    if (e != cudaSuccess) return e;
-    return launch_part_fine(p, bstart, sms, s);
-}
-
 template <int TYPE>
 cudaError_t slab_count_t(const EmitParams& p, int shift, int n_slabs, uint32_t* counts, cudaStream_t s) {
     k_slab_count<TYPE><<<p.n_cta, EMIT_THREADS, 0, s>>>(p, shift, n_slabs, counts);

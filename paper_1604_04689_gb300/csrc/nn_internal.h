@@ -254,8 +254,7 @@ cudaError_t launch_chunk_advance(int64_t* base, const uint32_t* etot, const uint
 cudaError_t launch_slab_count(const EmitParams& p, int shift, int n_slabs, uint32_t* counts, cudaStream_t s);
 cudaError_t launch_hist(const EmitParams& p, size_t smem, cudaStream_t s);
 cudaError_t launch_part(const EmitParams& p, cudaStream_t s);
-cudaError_t launch_part_sorted(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s);
-// the two passes of launch_part_sorted on their own (the fine pass only when cshift > 0)
+// the tile-sorted partition's two passes (the fine one only when cshift > 0)
 cudaError_t launch_part_coarse(const EmitParams& p, cudaStream_t s);
 int coarse_ctas_per_sm(int type);
 cudaError_t launch_part_fine(const EmitParams& p, const uint32_t* bstart, int sms, cudaStream_t s);
