@@ -122,6 +122,9 @@ nn_status nn_query(nn_handle* h, const nn_mesh* mesh, int want, size_t* ws_bytes
  * bucket_threads: 128 or 256 threads per bucket CTA; bucket_ctas_per_sm: 1..8
  * bucket CTAs sharing an SM (sets the shared memory per CTA, which caps the
  * bucket width).  Results never depend on tuning, only speed and workspace size.
+ * A mesh small enough to be built without a partition (nn_plan_info) takes sb,
+ * when that leaves it few enough buckets, and not bucket_threads;
+ * bucket_ctas_per_sm has it partitioned.
  * nn_set_tuning(h, NULL) restores the automatic choice. */
 typedef struct {
     int32_t sb;
@@ -155,9 +158,11 @@ nn_status nn_element_neighbors(nn_handle* h, const nn_mesh* mesh, const nn_csr* 
  * element walk, [3] bytes per incidence record, [4] minimum workspace bytes,
  * [5] CTAs of the bucket pass, [6] threads per bucket CTA, [7] shared memory
  * per bucket CTA, [8] partition mode (-1 scattered, 0 one sorted pass, k > 0
- * coarse + fine sorted passes with 2^k buckets per coarse region; the mode of
- * a partitioned build: small meshes are built without), [9] kernels one build
- * launches. */
+ * coarse + fine sorted passes with 2^k buckets per coarse region), [9] kernels
+ * one build launches.  [2], [3] and [5] to [8] are those of a partitioned
+ * build; small meshes (up to 65,536 incidences, mixed ones 32,768, and a bucket
+ * per SM) are built without: one CTA per bucket, of its own size, in 3 kernels
+ * (2 without node rows). */
 nn_status nn_plan_info(nn_handle* h, const nn_mesh* mesh, int want, int64_t* info, int n);
 
 /* Neighbor nodes of every node (Sec. 2.1.1, Sec. 2.2.1) into *out. */
