@@ -1030,8 +1030,8 @@ def whole_job_value(n_elems, steps, world, total_ms):
 def launches_per_build(plan, want="both"):
     """Kernels one build launches, from its plan; of a plan that does not say:
     histogram, offsets, partition (one pass, or coarse + fine when the buckets
-    span more than 256 coarse digits), bucket, and for node rows their
-    placement (scan + copy)."""
+    span more than 256 coarse digits), bucket (one launch), and for node rows
+    their placement (scan + copy)."""
     if "kernels" in plan:
         return plan["kernels"]
     return 3 + (2 if plan["partition"] > 0 else 1) + (2 if want in ("both", "nodes") else 0)
@@ -1039,9 +1039,9 @@ def launches_per_build(plan, want="both"):
 
 # the sources that compile the single-mesh build's kernels and their launch
 # plan: traffic counters taken on other sources no longer describe them
-MEASURED_SOURCES = ("nn_api.cu", "nn_bucket.cu", "nn_bucket.cuh", "nn_bucket16.cu",
-                    "nn_bucket32.cu", "nn_bucket_direct.cu", "nn_bucket_direct32.cu", "nn_bulk.cuh", "nn_compact.cu", "nn_device.cuh", "nn_emit.cu",
-                    "nn_internal.h")
+MEASURED_SOURCES = ("nn_api.cu", "nn_bucket.cu", "nn_bucket.cuh", "nn_bucket16.cu", "nn_bucket32.cu",
+                    "nn_bucket_direct.cu", "nn_bucket_direct32.cu", "nn_bucket_rest.cu", "nn_bulk.cuh", "nn_compact.cu",
+                    "nn_device.cuh", "nn_emit.cu", "nn_internal.h")
 
 
 def source_digest():

@@ -9,10 +9,12 @@
 // triangles borders both tets.
 //
 // A mesh of one type is matched node by node (k_adj_match): the elements
-// around a node are held by the lanes of a group, and a lane compares the
-// faces of its element that contain the node with every other element there.
-// Each face is settled once, at its smallest node, and what lies across it
-// goes into one slot per element and face; the rows are the sorted slots.
+// around a node are held by the lanes of a group.  Each face is settled once,
+// at its smallest node: tets put the faces whose smallest node this is into a
+// small hash table per warp, the other types compare the faces of a lane's
+// element that contain the node with every other element there (as tets do in
+// rows longer than a warp).  What lies across a face goes into one slot per
+// element and face; the rows are the sorted slots.
 // Elements for which one slot per face is not enough (several elements across
 // a face, a face that lies in an element without being one of its faces,
 // repeated nodes, a node with very many elements) are flagged.  A flagged

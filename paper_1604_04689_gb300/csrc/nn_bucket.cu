@@ -1,5 +1,5 @@
-// The bucket pass with up to 8 slots per node, and the choice among the
-// variants by their register arrays.
+// The bucket pass with up to 8 slots per node, the choice among the variants
+// by their register arrays, and its two launches.
 #include "nn_bucket.cuh"
 
 namespace nn {

@@ -1,5 +1,5 @@
 // Bulk asynchronous copies into shared memory and their mbarriers (used by
-// the fine partition pass and the bucket pass).
+// the fine partition pass).
 #pragma once
 
 #include "nn_device.cuh"
