@@ -35,7 +35,7 @@
 // on 30 % of their mesh's node ids 1100 -> 333 us, a fan of 20,000 triangles
 // 25.8 -> 1.2 ms.
 //
-// What bounds it: instructions (issue slots 65 % busy on hexes), then
+// What bounds it: instructions (issue slots 63 % busy on hexes), then
 // instruction fetch where the networks are long (tets) and shared-memory
 // stores.  Before, records were staged in shared memory, counted, scanned and
 // gathered by index twice at 16 warps per SM (issue 31-49 %), and tets went
